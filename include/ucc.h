@@ -93,7 +93,12 @@ typedef struct {
                            determinants remain after a factor keep the n_cut of
                            largest |c| (ties: smaller key).  0 = off. */
   int64_t max_entries;  /* hard cap on stored determinants, 0 = device memory */
-  int32_t probe_width;  /* lanes per hash probe: 1, 2, 4 or 8; 0 = autotuned */
+  int32_t probe_width;  /* lanes per hash probe: 1, 2, 4 or 8; 0 = autotuned.
+                           Tables that fit a thread-block cluster's shared
+                           memory run resident in it, a whole run of factors
+                           per launch, unless probe_width, max_entries or
+                           rebuild_test_regions is set (their results are the
+                           same) */
   int32_t checkpoint_stride; /* gradient: factors between snapshots of psi; 0 =
                                 one segment while the kill tape fits its
                                 budget, else ceil(sqrt(K)) */
@@ -123,8 +128,8 @@ typedef struct {
   int32_t energy_test_buffer_records; /* test only: cap on the records one
                                          round of the bucketed energy holds
                                          (0 = sized by the library) */
-  int32_t rebuild_test_regions; /* test only: hash builds by regions (one-word
-                                   keys): 0 = for tables of at least 2^20
+  int32_t rebuild_test_regions; /* test only: one launch per factor, and hash
+                                   builds by regions (one-word keys): 0 = for tables of at least 2^20
                                    slots (and bulk re-insertions of at least
                                    one record per eight slots), 1 = never,
                                    2 = for every table of at least 8,192 slots
@@ -227,7 +232,9 @@ ucc_status ucc_get_stats(const ucc_ctx* ctx, ucc_stats* out);
 
 /* Energies and gradients of n_jobs independent contexts (molecules or theta
  * vectors of uneven size): E[j] and grads[j][0..n_exc_j) (host pointers;
- * grads may be NULL for energy only).  Every job whose table can be sized up
+ * grads may be NULL for energy only).  Jobs of one-word keys whose table fits
+ * a thread-block cluster's shared memory run resident, a cluster per job, all
+ * of them in one launch per pass.  Every other job whose table can be sized up
  * front (three times its determinant sector, or three times its n_max when
  * its Methods-section cut can fire; at most 2^22 entries; keys of one word)
  * runs in one cooperative

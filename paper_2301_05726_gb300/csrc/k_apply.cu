@@ -375,17 +375,19 @@ __global__ void __launch_bounds__(kThreads) k_export(TableT<KT> t, unsigned long
   }
 }
 
-// psi = {HF: 1.0}; the slots are already zero.
+// psi = {HF: 1.0}; with_hash: in the hash too, whose slots are already zero.
 template <class KT>
-__global__ void k_reset(TableT<KT> t, KT hf) {
+__global__ void k_reset(TableT<KT> t, KT hf, bool with_hash) {
   Counters* c = t.cnt;
   t.keys[0] = hf;
   t.amps[0] = 1.0;
   if (t.born) t.born[0] = BORN_INITIAL;
-  const unsigned long long s = home_slot(t, hf);
-  t.slots[s].key = hf;
-  t.slots[s].idx = 0;
-  filter_add(t, hf);
+  if (with_hash) {
+    const unsigned long long s = home_slot(t, hf);
+    t.slots[s].key = hf;
+    t.slots[s].idx = 0;
+    filter_add(t, hf);
+  }
   c->n_tail = 1;
   c->n_scan = 1;
   c->stop_k = -1;
@@ -394,8 +396,8 @@ __global__ void k_reset(TableT<KT> t, KT hf) {
 }  // namespace
 
 template <class KT>
-cudaError_t launch_reset(const TableT<KT>& t, KT hf, cudaStream_t st) {
-  k_reset<KT><<<1, 1, 0, st>>>(t, hf);
+cudaError_t launch_reset(const TableT<KT>& t, KT hf, bool with_hash, cudaStream_t st) {
+  k_reset<KT><<<1, 1, 0, st>>>(t, hf, with_hash);
   return cudaGetLastError();
 }
 
@@ -484,7 +486,7 @@ cudaError_t launch_export(const TableT<KT>& t, unsigned long long cap, KT* keys,
 }
 
 #define UCC_APPLY_INSTANTIATE(KT)                                                                                  \
-  template cudaError_t launch_reset<KT>(const TableT<KT>&, KT, cudaStream_t);                                      \
+  template cudaError_t launch_reset<KT>(const TableT<KT>&, KT, bool, cudaStream_t);                                      \
   template cudaError_t launch_forward<KT>(const TableT<KT>&, const FactorT<KT>*, int, double, unsigned int, int,   \
                                           const TapeT<KT>&, unsigned long long, int, int, cudaStream_t);           \
   template cudaError_t launch_compact<KT>(const TableT<KT>&, const TableT<KT>&, int, int, cudaStream_t);           \

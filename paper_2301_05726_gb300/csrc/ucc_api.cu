@@ -123,6 +123,9 @@ struct TableSet {
   // next rebuild waits for `clean` instead of clearing on the main stream.
   cudaEvent_t clean = nullptr;
   bool clean_pending = false;
+  // Whether cur's slot array and filter index its entries.  A resident pass
+  // leaves entries only; ensure_hash builds the hash when a kernel needs it.
+  bool hash_valid = true;
   void release() {
     cur.release();
     spare.release();
@@ -459,6 +462,7 @@ ucc_status finish_rebuild(ucc_ctx* c, TableSet& s, const TableT<KT>& to, unsigne
   CUDA_TRY(launch_finish_rebuild(to, expect, c->stream));
   c->launches += 1;
   std::swap(s.cur, s.spare);
+  s.hash_valid = true;
   s.cur.slots_clean = false;  // the live hash
   s.spare.slots_clean = false;  // the previous live hash, until cleared
   // After growth the old, smaller arrays are not reused: free them now.
@@ -577,6 +581,38 @@ void release_tape(ucc_ctx* c) {
   c->tape_cap = 0;
 }
 
+// Determinants in a problem's sector (fixed alpha and beta electron counts), saturating at 2^62.
+unsigned long long sector_bound(const ucc_ctx* c) {
+  auto comb = [](int n, int k) {
+    double r = 1.0;
+    for (int i = 1; i <= k; ++i) r = r * (double)(n - k + i) / (double)i;
+    return r;
+  };
+  const double d = comb(c->n_spatial, c->n_alpha) * comb(c->n_spatial, c->n_beta);
+  return d < 4.6e18 ? (unsigned long long)(d + 0.5) : 1ull << 62;
+}
+
+// Shape of the resident passes of a problem (k_resident.cu): for all its
+// tables where they fit a cluster's shared memory, else the largest shape,
+// for the factors at either end of a pass where the table is small.  False:
+// none, or options that speak of the launch-per-factor path (a fixed probe
+// width, an entry cap that its chunks check, the region-build test hook).
+bool resident_shape(const ucc_ctx* c, ResGeom* g, unsigned long long* bound) {
+  if (c->opt.rebuild_test_regions != 0 || c->opt.probe_width != 0 || c->opt.max_entries > 0) return false;
+  const int most = res_max_logC(c->kw);
+  if (most < 0) return false;
+  *bound = sector_bound(c);
+  unsigned long long need = *bound;
+  if (c->opt.n_max > 0) need = std::min(need, 2ull * (unsigned long long)c->opt.n_max);
+  *g = res_geometry(need, c->kw, most);
+  return true;
+}
+
+// Entries a table needs in global memory for what a resident pass can write back.
+unsigned long long resident_cap(const ResGeom& g, unsigned long long bound) {
+  return std::min<unsigned long long>((unsigned long long)g.L << g.logC, bound);
+}
+
 template <class KT>
 KT reference_key(const ucc_ctx* c) {
   KT hf = KeyOps<KT>::zero();
@@ -585,15 +621,37 @@ KT reference_key(const ucc_ctx* c) {
   return hf;
 }
 
-// psi = {reference: 1.0} in table s.
+// psi = {reference: 1.0} in table s, with room for min_cap entries; hashed
+// when with_hash.
 template <class KT>
-ucc_status reset_table(ucc_ctx* c, TableSet& s) {
-  if (s.cur.cap_n == 0) UCC_TRY(s.cur.allocate(1 << 12, slots_for(1 << 12)));
+ucc_status reset_table(ucc_ctx* c, TableSet& s, bool with_hash, unsigned long long min_cap = 0) {
+  min_cap = std::max<unsigned long long>(min_cap, s.cur.cap_n == 0 ? 1 << 12 : 0);
+  if (s.cur.cap_n < min_cap) UCC_TRY(s.cur.allocate(min_cap, slots_for(min_cap)));
   CUDA_TRY(cudaMemsetAsync(s.d_cnt, 0, sizeof(Counters), c->stream));
+  if (with_hash) {
+    CUDA_TRY(cudaMemsetAsync(s.cur.slots, 0, s.cur.n_slots * sizeof(SlotT<KT>), c->stream));
+    CUDA_TRY(cudaMemsetAsync(s.cur.filt, 0, s.cur.n_slots / 4 * sizeof(unsigned int), c->stream));
+  }
+  CUDA_TRY(launch_reset(c->template table<KT>(s), reference_key<KT>(c), with_hash, c->stream));
+  c->launches++;
+  s.hash_valid = with_hash;
+  return UCC_OK;
+}
+
+// The hash of table s, whose entries are distinct keys (a resident pass
+// leaves no dropped ones), if it is not there.
+template <class KT>
+ucc_status ensure_hash(ucc_ctx* c, TableSet& s) {
+  if (s.hash_valid) return UCC_OK;
   CUDA_TRY(cudaMemsetAsync(s.cur.slots, 0, s.cur.n_slots * sizeof(SlotT<KT>), c->stream));
   CUDA_TRY(cudaMemsetAsync(s.cur.filt, 0, s.cur.n_slots / 4 * sizeof(unsigned int), c->stream));
-  CUDA_TRY(launch_reset(c->template table<KT>(s), reference_key<KT>(c), c->stream));
+  CUDA_TRY(cudaMemcpyAsync(&s.d_cnt->new_n, &s.d_cnt->n_tail, sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
+                           c->stream));
+  CUDA_TRY(launch_rehash(c->template table<KT>(s), c->full_grid(), c->stream));
+  CUDA_TRY(cudaMemsetAsync(&s.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
   c->launches++;
+  s.cur.slots_clean = false;
+  s.hash_valid = true;
   return UCC_OK;
 }
 
@@ -608,9 +666,15 @@ ucc_status reset_tape(ucc_ctx* c, TableSet& s, int k0) {
 // Load a snapshot into table s (its previous contents are discarded).
 template <class KT>
 ucc_status load_snapshot(ucc_ctx* c, TableSet& s, const Snapshot& snap) {
-  const unsigned long long cap = std::max<unsigned long long>(4 * snap.n, 1 << 12);
+  unsigned long long cap = std::max<unsigned long long>(4 * snap.n, 1 << 12);
+  {
+    ResGeom g{};
+    unsigned long long bound = 0;
+    if (resident_shape(c, &g, &bound)) cap = std::max(cap, resident_cap(g, bound));
+  }
   if (cap >= kMaxEntries) return fail(UCC_ECAPACITY, "snapshot too large for one table");
   if (s.cur.cap_n < cap) UCC_TRY(s.cur.allocate(cap, slots_for(cap)));
+  s.hash_valid = true;
   CUDA_TRY(cudaMemsetAsync(s.d_cnt, 0, sizeof(Counters), c->stream));
   CUDA_TRY(cudaMemsetAsync(s.cur.slots, 0, s.cur.n_slots * sizeof(SlotT<KT>), c->stream));
   CUDA_TRY(cudaMemsetAsync(s.cur.filt, 0, s.cur.n_slots / 4 * sizeof(unsigned int), c->stream));
@@ -741,7 +805,102 @@ ucc_status ensure_room(ucc_ctx* c, TableSet& s, bool record) {
   return ensure_room_known<KT>(c, s, record, &h);
 }
 
-// Factors [k0, k1) on table s.  The last block of each factor flags a stop
+template <class KT>
+ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, double eps, unsigned long long bound, int k0, int k1) {
+  ResJob<KT> j{};
+  j.t = c->template table<KT>(s);
+  j.factors = c->template dfactors<KT>();
+  j.tape = c->template tape<KT>();
+  j.grad = c->d_grad;
+  j.eps = eps;
+  j.n_max = c->opt.n_max > 0 ? (unsigned long long)c->opt.n_max : 0ull;
+  j.n_cut = c->opt.n_cut > 0 ? (unsigned long long)c->opt.n_cut : 0ull;
+  j.bound = bound;
+  j.k0 = k0;
+  j.k1 = k1;
+  return j;
+}
+
+// More tape for a resident pass that holds h.tape_n records: twice as many
+// (few launches), or, past the call's budget, what the next factors need.
+ucc_status resident_tape(ucc_ctx* c, const Counters& h) {
+  const unsigned long long need = h.tape_n + 4ull * (h.n_tail - h.n_dead) + (1ull << 12);
+  if (c->tape_cap >= need && c->tape_cap >= 2ull * h.tape_n) return UCC_OK;
+  if (ensure_tape(c, std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
+  c->tape_over_budget = false;
+  cudaGetLastError();
+  return ensure_tape(c, need);
+}
+
+// What a resident forward launch left in the job's counters (its host mirror).
+void resident_account(ucc_ctx* c, const Counters& h) {
+  c->cut_total += (long long)h.res_cut;
+  c->stats.rebuilds += (long long)h.res_rebuilds;
+  c->stats.peak_entries = std::max<long long>(c->stats.peak_entries, (long long)h.res_peak);
+}
+
+// As many of the factors [*k, k1) as one cluster can hold, on table s, whose
+// counters the host mirror holds; *k moves to the first one left.
+template <class KT>
+ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, int* k, int k1) {
+  ResGeom g{};
+  unsigned long long bound = 0;
+  if (!resident_shape(c, &g, &bound) || s.cur.cap_n < resident_cap(g, bound)) return UCC_OK;
+  while (*k < k1) {
+    const unsigned long long live = s.h_cnt->n_tail - s.h_cnt->n_dead;
+    if (!res_room_host(std::min(2ull * live, bound), g)) return UCC_OK;
+    if (record) UCC_TRY(resident_tape(c, *s.h_cnt));
+    CUDA_TRY(cudaMemsetAsync(&s.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
+    CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
+    CUDA_TRY(launch_res_forward<KT>(resident_job<KT>(c, s, eps, bound, *k, k1), nullptr, 1, g, record ? 1 : 0,
+                                    c->stream));
+    CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
+    c->launches++;
+    c->stats.forward_launches++;
+    UCC_TRY(read_counters(c, s));
+    float ms = 0.f;
+    CUDA_TRY(cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]));
+    c->stats.forward_kernel_ms += ms;
+    const Counters& h = *s.h_cnt;
+    if (h.res_status == RES_ABORT || h.res_k == *k) return UCC_OK;  // nothing was applied
+    if (h.res_k < *k || h.res_k > k1) return fail(UCC_ECUDA, "invalid resume factor");
+    s.hash_valid = false;
+    resident_account(c, h);
+    *k = h.res_k;
+    if (h.res_status != RES_TAPE) return UCC_OK;
+  }
+  return UCC_OK;
+}
+
+// The reverse of the factors [k0, *k1) on table s as far as one cluster can
+// hold it; *k1 moves down to the first factor undone last.
+template <class KT>
+ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int* k1) {
+  ResGeom g{};
+  unsigned long long bound = 0;
+  if (!resident_shape(c, &g, &bound) || s.cur.cap_n < resident_cap(g, bound)) return UCC_OK;
+  if (!res_room_host(s.h_cnt->n_tail - s.h_cnt->n_dead, g)) return UCC_OK;
+  CUDA_TRY(cudaMemsetAsync(&s.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
+  CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
+  CUDA_TRY(launch_res_reverse<KT>(resident_job<KT>(c, s, 0.0, bound, k0, *k1), nullptr, 1, g, c->stream));
+  CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
+  c->launches++;
+  c->stats.reverse_launches++;
+  UCC_TRY(read_counters(c, s));
+  float ms = 0.f;
+  CUDA_TRY(cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]));
+  c->stats.reverse_kernel_ms += ms;
+  const Counters& h = *s.h_cnt;
+  if (h.res_status == RES_ABORT) return UCC_OK;
+  if (h.res_k < k0 || h.res_k > *k1) return fail(UCC_ECUDA, "invalid resume factor");
+  s.hash_valid = false;
+  c->stats.reverse_compactions += (long long)h.res_rebuilds;
+  *k1 = h.res_k;
+  return UCC_OK;
+}
+
+// Factors [k0, k1) on table s: resident in one cluster while the table is
+// small, then one launch per factor.  The last block of each factor flags a stop
 // when the next factor might not fit or when the Methods-section cut is due;
 // later launches in the chunk then skip, and the host cuts / grows and
 // resumes at the flagged factor.  Chunks shrink when stops come often.
@@ -749,9 +908,17 @@ template <class KT>
 ucc_status run_factors(ucc_ctx* c, TableSet& s, double eps, bool record, int k0, int k1) {
   const unsigned long long n_max = c->opt.n_max > 0 ? (unsigned long long)c->opt.n_max : 0ull;
   UCC_TRY(read_counters(c, s));
+  int k = k0;
+  UCC_TRY(resident_forward<KT>(c, s, eps, record, &k, k1));
+  if (k == k1) return UCC_OK;
+  UCC_TRY(ensure_hash<KT>(c, s));
+  if (k > k0) {
+    Counters known = *s.h_cnt;  // room for the next factor, as after every stop
+    UCC_TRY(ensure_room_known<KT>(c, s, record, &known));
+    *s.h_cnt = known;
+  }
   unsigned long long n_known = s.h_cnt->n_tail;
   int chunk = 64;
-  int k = k0;
   // Growth per factor of the live entries and of the table's tail, from the
   // last chunk: a chunk is sized to end just past the factor expected to
   // stop it (a cut or a table that needs room), so few launches after a stop
@@ -860,6 +1027,15 @@ int segment_stride(const ucc_ctx* c) {
   return std::max(1, c->K);
 }
 
+// The reference state in table s, sized and (not) hashed for the path that runs first.
+template <class KT>
+ucc_status reset_for_run(ucc_ctx* c, TableSet& s) {
+  ResGeom g{};
+  unsigned long long bound = 0;
+  const bool resident = c->K > 0 && resident_shape(c, &g, &bound);
+  return reset_table<KT>(c, s, !resident, resident ? resident_cap(g, bound) : 0ull);
+}
+
 template <class KT>
 ucc_status run_forward(ucc_ctx* c, double eps, bool record) {
   if (!(eps >= 0.0) || std::isinf(eps)) return fail(UCC_EINVAL, "eps must be finite and >= 0");
@@ -867,7 +1043,7 @@ ucc_status run_forward(ucc_ctx* c, double eps, bool record) {
   c->cut_total = 0;
   c->entropy_on = !record && c->opt.record_entropy != 0;
   c->have_entropy = false;
-  UCC_TRY(reset_table<KT>(c, s));
+  UCC_TRY(reset_for_run<KT>(c, s));
   CUDA_TRY(cudaEventRecord(c->ev[0], c->stream));
   if (!record) {
     UCC_TRY(run_factors<KT>(c, s, eps, false, 0, c->K));
@@ -1030,6 +1206,7 @@ ucc_status run_energy(ucc_ctx* c, double* E, double* norm2) {
   unsigned long long records = 0;
   if (c->opt.energy_route != 1) UCC_TRY(energy_by_buckets<KT>(c, s, in, &bucketed, &records));
   if (!bucketed) {
+    UCC_TRY(ensure_hash<KT>(c, s));
     CUDA_TRY(launch_sigma(c->template table<KT>(s), in, grid, c->stream));
     c->launches += 2;
   }
@@ -1065,6 +1242,17 @@ ucc_status reverse_segment(ucc_ctx* c, TableSet& s, int k0, int k1) {
   CUDA_TRY(cudaMemcpyAsync(off.data(), c->t_off + k0, off.size() * sizeof(unsigned long long),
                            cudaMemcpyDeviceToHost, c->stream));
   UCC_TRY(read_counters(c, s));
+  {
+    int k = k1;
+    UCC_TRY(resident_reverse<KT>(c, s, k0, &k));
+    if (k == k0) {
+      c->stats.reverse_pairs += (long long)s.h_cnt->rev_pairs;
+      c->stats.reverse_scanned += (long long)s.h_cnt->rev_scanned;
+      return UCC_OK;
+    }
+    k1 = k;
+  }
+  UCC_TRY(ensure_hash<KT>(c, s));
   const int grid_full = c->full_grid();
   unsigned long long bound = s.h_cnt->n_tail;
   int grid = (int)std::min<unsigned long long>((unsigned long long)grid_full, (bound * 2 + 255) / 256);
@@ -1189,7 +1377,7 @@ ucc_status run_gradient_once(ucc_ctx* c, double eps, double* E, double* grad_out
       TableSet& from = c->ts[c->main];
       TableSet& work = c->ts[1 - c->main];
       if (j == 0) {
-        UCC_TRY(reset_table<KT>(c, work));
+        UCC_TRY(reset_for_run<KT>(c, work));
       } else {
         UCC_TRY(load_snapshot<KT>(c, work, c->snaps[j]));
       }
@@ -1200,6 +1388,7 @@ ucc_status run_gradient_once(ucc_ctx* c, double eps, double* E, double* grad_out
       c->stats.recompute_rotations += (long long)work.h_cnt->rotations;
       c->stats.recompute_created += (long long)work.h_cnt->created;
       tape_peak = std::max<long long>(tape_peak, (long long)work.h_cnt->tape_n);
+      UCC_TRY(ensure_hash<KT>(c, from));
       CUDA_TRY(launch_transfer_lambda(c->template table<KT>(work), c->template table<KT>(from), grid_full, c->stream));
       c->launches++;
       c->main = 1 - c->main;
@@ -1373,6 +1562,224 @@ cudaGraphExec_t capture_one(cudaStream_t st, F launch) {
   return ex;
 }
 
+// One job by itself through the one-job path.
+ucc_status run_alone(ucc_ctx* c, double eps, double* E, double* grad) {
+  if (grad)
+    return c->wide ? run_gradient<Key128>(c, eps, E, grad, 0) : run_gradient<unsigned long long>(c, eps, E, grad, 0);
+  c->launches = 0;
+  drop_timings(c);
+  c->stats = ucc_stats{};
+  if (c->wide) {
+    UCC_TRY(run_forward<Key128>(c, eps, false));
+    return run_energy<Key128>(c, E, nullptr);
+  }
+  UCC_TRY(run_forward<unsigned long long>(c, eps, false));
+  return run_energy<unsigned long long>(c, E, nullptr);
+}
+
+// Whether every table of job c fits a cluster (one-word keys: the batched
+// energy's), under the batch options that speak of the persistent launches.
+bool batch_resident_ok(const ucc_ctx* c, const ucc_options& first) {
+  if (c->wide || c->K == 0 || first.batch_tiles != 0 || first.batch_test_skip_block != 0) return false;
+  ResGeom g{};
+  unsigned long long bound = 0;
+  if (!resident_shape(c, &g, &bound)) return false;
+  if (c->opt.n_max > 0) bound = std::min(bound, 2ull * (unsigned long long)c->opt.n_max);
+  return res_fits(bound, 1, res_max_logC(1)) && c->opt.checkpoint_stride == 0 && c->opt.record_entropy == 0;
+}
+
+// The batched path for small tables: a cluster per job runs all its factors
+// in shared memory (k_resident.cu), every job in one launch; the energy of all
+// jobs in one launch; the reverse sweeps in one launch.  A job that a cluster
+// could not hold to the end is left to the one-job path (*alone).
+ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, double eps, double* E,
+                          double* const* grads, std::vector<int>* alone) {
+  using KT = unsigned long long;
+  const int n = (int)idx.size();
+  ucc_ctx* c0 = jobs[idx[0]];
+  cudaStream_t st = c0->stream;
+  bool record = false;
+  for (int x : idx) record |= grads && grads[x];
+  // The longest jobs first: they start first and the short ones fill in.
+  std::vector<int> order(idx);
+  auto most_entries = [&](const ucc_ctx* c) {
+    const unsigned long long sector = sector_bound(c);
+    return c->opt.n_max > 0 ? std::min(sector, 2ull * (unsigned long long)c->opt.n_max) : sector;
+  };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    const ucc_ctx *x = jobs[a], *y = jobs[b];
+    return (double)x->K * (4000.0 + (double)most_entries(x)) > (double)y->K * (4000.0 + (double)most_entries(y));
+  });
+  unsigned long long bound = 1;
+  for (int x : order) bound = std::max(bound, most_entries(jobs[x]));
+  // Clusters of eight keep twice as many jobs in flight as clusters of
+  // sixteen, which pays from ten jobs on (nine large clusters fill the GPU).
+  int max_logC = res_max_logC(1);
+  if (n > 9 && max_logC > 3 && res_fits(bound, 1, 3)) max_logC = 3;
+  const ResGeom g = res_geometry(bound, 1, max_logC);
+  ResJob<KT>* d_jobs = nullptr;
+  JobView* d_view = nullptr;
+  JobState* d_js = nullptr;
+  BatchHeader* d_bh = nullptr;
+  auto release = [&]() {
+    dfree(d_jobs);
+    dfree(d_view);
+    dfree(d_js);
+    dfree(d_bh);
+  };
+  auto run = [&]() -> ucc_status {
+    UCC_TRY(dalloc(&d_jobs, n));
+    UCC_TRY(dalloc(&d_view, n));
+    UCC_TRY(dalloc(&d_js, n));
+    UCC_TRY(dalloc(&d_bh, 1));
+    for (int x : order) {
+      ucc_ctx* c = jobs[x];
+      c->launches = 0;
+      drop_timings(c);
+      c->stats = ucc_stats{};
+      c->cut_total = 0;
+      c->tape_budget = 0;
+      c->main = 0;
+      c->entropy_on = false;
+      c->have_entropy = false;
+      c->have_psi = c->have_sigma = false;
+      UCC_TRY(settle_spare(c, c->ts[0]));
+      UCC_TRY(reset_table<KT>(c, c->ts[0], false, resident_cap(g, sector_bound(c))));
+      if (record) UCC_TRY(reset_tape(c, c->ts[0], 0));
+      *c->ts[0].h_cnt = Counters{};
+    }
+    // Counters of the jobs in `which`, one synchronisation for all.
+    auto read_all = [&](const std::vector<int>& which) -> ucc_status {
+      for (int x : which) {
+        TableSet& s = jobs[x]->ts[0];
+        CUDA_TRY(cudaMemcpyAsync(s.h_cnt, s.d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+      }
+      CUDA_TRY(cudaStreamSynchronize(st));
+      for (int x : which) UCC_TRY(check_device_error(*jobs[x]->ts[0].h_cnt));
+      return UCC_OK;
+    };
+    std::vector<ResJob<KT>> hj(n);
+    auto upload = [&](const std::vector<int>& which, bool reverse) -> ucc_status {
+      for (size_t y = 0; y < which.size(); ++y) {
+        ucc_ctx* c = jobs[which[y]];
+        hj[y] = resident_job<KT>(c, c->ts[0], eps, sector_bound(c), reverse ? 0 : c->ts[0].h_cnt->res_k, c->K);
+      }
+      CUDA_TRY(cudaMemcpyAsync(d_jobs, hj.data(), which.size() * sizeof(ResJob<KT>), cudaMemcpyHostToDevice, st));
+      return UCC_OK;
+    };
+    // Forward: again for the jobs that wait for more tape.
+    CUDA_TRY(cudaEventRecord(c0->ev[0], st));
+    std::vector<int> todo(order), done;
+    while (!todo.empty()) {
+      UCC_TRY(upload(todo, false));
+      CUDA_TRY(launch_res_forward<KT>(hj[0], d_jobs, (int)todo.size(), g, record ? 1 : 0, st));
+      UCC_TRY(read_all(todo));
+      std::vector<int> more;
+      for (int x : todo) {
+        ucc_ctx* c = jobs[x];
+        const Counters& h = *c->ts[0].h_cnt;
+        c->launches++;
+        c->stats.forward_launches++;
+        c->ts[0].hash_valid = false;
+        if (h.res_status == RES_DONE && h.res_k == c->K) {
+          resident_account(c, h);
+          done.push_back(x);
+        } else if (h.res_status == RES_TAPE) {
+          resident_account(c, h);
+          UCC_TRY(resident_tape(c, h));
+          more.push_back(x);
+        } else {
+          alone->push_back(x);
+        }
+      }
+      todo.swap(more);
+    }
+    CUDA_TRY(cudaEventRecord(c0->ev[1], st));
+    if (done.empty()) return UCC_OK;
+    // (the jobs that finished late go last: keep the order of the first launch)
+    std::vector<int> jobs_in;
+    for (int x : order)
+      if (std::find(done.begin(), done.end(), x) != done.end()) jobs_in.push_back(x);
+    const int m = (int)jobs_in.size();
+    std::vector<JobView> hv(m);
+    std::vector<JobState> hs(m);
+    for (int y = 0; y < m; ++y) {
+      ucc_ctx* c = jobs[jobs_in[y]];
+      fill_forward_stats(c, *c->ts[0].h_cnt);
+      c->stats.tape_entries = (long long)c->ts[0].h_cnt->tape_n;
+      c->stats.capacity_entries = (long long)c->ts[0].cur.cap_n;
+      c->stats.hash_slots = (long long)c->ts[0].cur.n_slots;
+      UCC_TRY(ensure_hash<KT>(c, c->ts[0]));
+      JobView v{};
+      v.t = c->template table<KT>(c->ts[0]);
+      v.factors = c->template dfactors<KT>();
+      v.in.h = c->d_h;
+      v.in.g = c->d_g;
+      v.in.n = c->n_spatial;
+      v.in.n_so = c->n_so;
+      v.grad = c->d_grad;
+      v.K = c->K;
+      hv[y] = v;
+      hs[y] = JobState{};
+    }
+    CUDA_TRY(cudaMemcpyAsync(d_view, hv.data(), m * sizeof(JobView), cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(d_js, hs.data(), m * sizeof(JobState), cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemsetAsync(d_bh, 0, sizeof(BatchHeader), st));
+    CUDA_TRY(launch_batch_layout(d_view, d_js, m, d_bh, st));
+    CUDA_TRY(cudaEventRecord(c0->ev[2], st));
+    CUDA_TRY(launch_sigma_batch(d_view, d_js, m, d_bh, c0->full_grid(), st));
+    CUDA_TRY(cudaEventRecord(c0->ev[3], st));
+    if (record) {
+      CUDA_TRY(launch_lambda_init_batch(d_view, d_js, m, d_bh, c0->full_grid(), st));
+      UCC_TRY(upload(jobs_in, true));
+      CUDA_TRY(cudaEventRecord(c0->ev[4], st));
+      CUDA_TRY(launch_res_reverse<KT>(hj[0], d_jobs, m, g, st));
+      CUDA_TRY(cudaEventRecord(c0->ev[5], st));
+    }
+    CUDA_TRY(cudaMemcpyAsync(hs.data(), d_js, m * sizeof(JobState), cudaMemcpyDeviceToHost, st));
+    UCC_TRY(read_all(jobs_in));
+    float ms[3] = {0.f, 0.f, 0.f};
+    CUDA_TRY(cudaEventElapsedTime(&ms[0], c0->ev[0], c0->ev[1]));
+    CUDA_TRY(cudaEventElapsedTime(&ms[1], c0->ev[2], c0->ev[3]));
+    if (record) CUDA_TRY(cudaEventElapsedTime(&ms[2], c0->ev[4], c0->ev[5]));
+    for (int y = 0; y < m; ++y) {
+      const int x = jobs_in[y];
+      ucc_ctx* c = jobs[x];
+      const Counters& h = *c->ts[0].h_cnt;
+      c->launches += record ? 5 : 3;
+      if (record && !(h.res_status == RES_DONE && h.res_k == 0)) {
+        alone->push_back(x);
+        continue;
+      }
+      E[x] = hs[y].e_num / hs[y].norm2 + c->e_nuc;
+      if (record && grads[x])
+        CUDA_TRY(cudaMemcpyAsync(grads[x], c->d_grad, c->K * sizeof(double), cudaMemcpyDeviceToHost, st));
+      c->stats.sigma_probes = (long long)h.sig_probes;
+      c->stats.sigma_hits = (long long)h.sig_hits;
+      c->stats.reverse_pairs = (long long)h.rev_pairs;
+      c->stats.reverse_scanned = (long long)h.rev_scanned;
+      c->stats.reverse_compactions = record ? (long long)h.res_rebuilds : 0;
+      c->stats.reverse_launches = record ? 1 : 0;
+      c->stats.probe_width = 1;
+      c->stats.batch_tiles = 1;
+      c->stats.kernel_launches = c->launches;
+      c->have_psi = !record;
+      c->have_sigma = !record;
+    }
+    c0->stats.apply_ms = ms[0];
+    c0->stats.energy_ms = ms[1];
+    c0->stats.reverse_ms = ms[2];
+    CUDA_TRY(cudaStreamSynchronize(st));
+    return UCC_OK;
+  };
+  const ucc_status s = run();
+  if (s != UCC_OK) cudaStreamSynchronize(st);  // nothing in flight reads the arrays released here
+  const std::string msg = g_last_error;
+  release();
+  g_last_error = msg;
+  return s;
+}
+
 // Persistent-batch tuning: (probe width, tiles per warp visit) per batch shape,
 // chosen by timing the first steps of the forward pass with each candidate.
 std::mutex g_btune_mutex;
@@ -1476,7 +1883,7 @@ ucc_status batch_persistent(const std::vector<int>& idx, ucc_ctx* const* jobs, d
       if (ts.cur.cap_n != cap || ts.cur.n_slots != ns) UCC_TRY(ts.cur.allocate(cap, ns));
       if (ts.spare.cap_n != cap || ts.spare.n_slots != ns) UCC_TRY(ts.spare.allocate(cap, ns));
       c->main = 0;
-      UCC_TRY(reset_table<unsigned long long>(c, ts));
+      UCC_TRY(reset_table<unsigned long long>(c, ts, true));
       if (record) UCC_TRY(reset_tape(c, ts, 0));
       hs[x] = JobState{};
       hs[x].stop = -1;
@@ -1921,31 +2328,20 @@ ucc_status ucc_batch_run(int n_jobs, ucc_ctx* const* jobs, double eps, double* E
       return fail(UCC_EINVAL, "batched jobs must share one device and one stream");
   }
   CUDA_TRY(cudaSetDevice(jobs[0]->device));
-  // Jobs whose table cannot be sized up front (no cut and a large sector)
-  // run one by one; the rest share the persistent launches.
-  std::vector<int> together;
+  // Jobs whose table fits a cluster's shared memory run resident; jobs whose
+  // table cannot be sized up front (no cut and a large sector) run one by
+  // one; the rest share the persistent launches.
+  std::vector<int> together, resident, alone;
   for (int j = 0; j < n_jobs; ++j) {
-    ucc_ctx* c = jobs[j];
-    if (batch_capacity(c) == 0 || together.size() >= (size_t)kMaxBatchJobs) {
-      if (grads && grads[j]) {
-        UCC_TRY(c->wide ? run_gradient<Key128>(c, eps, &E[j], grads[j], 0)
-                        : run_gradient<unsigned long long>(c, eps, &E[j], grads[j], 0));
-      } else {
-        c->launches = 0;
-        drop_timings(c);
-        c->stats = ucc_stats{};
-        if (c->wide) {
-          UCC_TRY(run_forward<Key128>(c, eps, false));
-          UCC_TRY(run_energy<Key128>(c, &E[j], nullptr));
-        } else {
-          UCC_TRY(run_forward<unsigned long long>(c, eps, false));
-          UCC_TRY(run_energy<unsigned long long>(c, &E[j], nullptr));
-        }
-      }
-    } else {
+    if (batch_resident_ok(jobs[j], jobs[0]->opt) && resident.size() < (size_t)kMaxBatchJobs)
+      resident.push_back(j);
+    else if (batch_capacity(jobs[j]) == 0 || together.size() >= (size_t)kMaxBatchJobs)
+      alone.push_back(j);
+    else
       together.push_back(j);
-    }
   }
+  if (!resident.empty()) UCC_TRY(batch_resident(resident, jobs, eps, E, grads, &alone));
+  for (int j : alone) UCC_TRY(run_alone(jobs[j], eps, &E[j], grads ? grads[j] : nullptr));
   if (together.empty()) return UCC_OK;
   return batch_together(together, jobs, eps, E, grads);
 }

@@ -59,6 +59,19 @@ struct Counters {
   unsigned long long err_key; // the key involved in it
   double e_num, norm2;        // <psi|H|psi>, <psi|psi> of the last energy pass
   double entropy;             // running Eq. 6 entropy of the stored state (when recorded)
+  // Result of the last resident launch (ResStatus; next factor; its cuts,
+  // rebuilds and largest entry count).
+  int res_status, res_k;
+  unsigned long long res_cut;
+  unsigned int res_rebuilds, res_peak;
+};
+
+// How a resident launch ended.
+enum ResStatus : int {
+  RES_DONE = 1,   // every factor asked for
+  RES_FULL = 2,   // before factor res_k (forward) or below it (reverse): the next one might not fit
+  RES_TAPE = 3,   // forward, before factor res_k: more kill tape is needed
+  RES_ABORT = 4   // a CTA's share outgrew its arrays: nothing was written back
 };
 
 // Where a consistency error was raised (Counters::err_site, first one wins).
@@ -150,6 +163,25 @@ struct __align__(32) SigRecT {
 };
 static_assert(sizeof(SigRecT<unsigned long long>) == 32, "record is one sector");
 
+// Shape of a resident launch (k_resident.cu): 2^logC CTAs a cluster, each with
+// room for L entries and 2^logB hash buckets of four slots.
+struct ResGeom {
+  int logC, L, logB;
+};
+
+// One job of a resident launch: factors [k0, k1) of a table that holds at most
+// `bound` determinants (its sector).
+template <class KT>
+struct ResJob {
+  TableT<KT> t;
+  const FactorT<KT>* factors;
+  TapeT<KT> tape;
+  double* grad;
+  double eps;
+  unsigned long long n_max, n_cut, bound;  // the cut (n_max 0: none)
+  int k0, k1;
+};
+
 // Radix-selection state of the N_MAX / N_CUT truncation.
 struct SelectState {
   unsigned long long prefix, target;          // |c| bits of the threshold, rank left inside it
@@ -236,7 +268,7 @@ constexpr unsigned int BORN_INITIAL = 0xFFFFFFFFu;  // the reference determinant
 // The single-problem path is built for one-word keys (KT = unsigned long
 // long, up to 64 spin-orbitals) and two-word keys (KT = Key128, up to 128).
 template <class KT>
-cudaError_t launch_reset(const TableT<KT>& t, KT hf, cudaStream_t st);
+cudaError_t launch_reset(const TableT<KT>& t, KT hf, bool with_hash, cudaStream_t st);
 template <class KT>
 cudaError_t launch_forward(const TableT<KT>& t, const FactorT<KT>* factors, int k, double eps, unsigned int stamp,
                            int record, const TapeT<KT>& tape, unsigned long long n_max, int probe_width, int grid,
@@ -340,6 +372,21 @@ cudaError_t launch_persist_reverse(JobView* jobs, JobState* js, int n_jobs, Batc
                                    int tiles, cudaStream_t st);
 // The persistent kernels' grid (blocks resident at once) on the current device.
 int persist_grid(int record, int probe_width, int reverse);
+// Resident passes: a cluster per job runs all its factors in shared memory.
+// res_geometry: the shape for tables of at most `bound` entries (clusters of at
+// most 2^max_logC CTAs); res_fits: whether any shape holds them.  many (n_jobs
+// of them, device memory) or, when null, the single job `one`.
+ResGeom res_geometry(unsigned long long bound, int key_words, int max_logC);
+bool res_fits(unsigned long long bound, int key_words, int max_logC);
+bool res_room_host(unsigned long long bound, const ResGeom& g);  // ... whether shape g does
+// Largest cluster (log2 of its CTAs) the current device runs these kernels in; -1: none.
+int res_max_logC(int key_words);
+template <class KT>
+cudaError_t launch_res_forward(const ResJob<KT>& one, const ResJob<KT>* many, int n_jobs, const ResGeom& g,
+                               int record, cudaStream_t st);
+template <class KT>
+cudaError_t launch_res_reverse(const ResJob<KT>& one, const ResJob<KT>* many, int n_jobs, const ResGeom& g,
+                               cudaStream_t st);
 // Message returned by ucc_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

@@ -132,24 +132,17 @@ __device__ __forceinline__ void link_from_slot(const TableT<KT>& t, KT key, unsi
   raise_error(t.cnt, ERR_PROBE_BOUND);
 }
 
-// DEFER: created entries are appended unlinked (link_appended runs after the
-// step); otherwise they are hashed at once.
-template <bool RECORD, bool DEFER = false, class KT>
-__device__ __forceinline__ void forward_resolve(const TableT<KT>& t, const FactorT<KT>& f, int k, double eps,
-                                                unsigned int stamp, const TapeT<KT>& tape, unsigned long long i, KT X,
-                                                double cX, bool ex, const Lookup& r, StepCounts& sc) {
-  const KT Y = X ^ (f.occ | f.vir);
-  const bool partner_live = (r.state == ALIVE);
-  if (!ex && (partner_live || r.state == DEAD_NOW)) return;  // E's thread owns the pair
-  if (ex && r.state == DEAD_NOW) {
-    raise_consistency(t.cnt, SITE_PAIR_OWNER);
-    return;
-  }
-  const KT E = ex ? X : Y;
+// The rotation of one linked pair seen from its stored member X (amplitude cX;
+// ex = X is the excited member E): the new amplitudes of X and of its partner
+// Y, whose amplitude cY counts only when partner_live.
+template <class KT>
+__device__ __forceinline__ void rotate_member(const FactorT<KT>& f, KT X, double cX, bool ex, bool partner_live,
+                                              double cY, double& nX, double& nY) {
+  const KT E = ex ? X : X ^ (f.occ | f.vir);
   const int parity = (KeyOps<KT>::popc(E & f.pmask) + f.pconst) & 1;
   const double ss = neg_if(f.s, parity);  // s * sin(theta), exact
   const double cE = ex ? cX : 0.0;
-  const double cD = ex ? (partner_live ? r.amp : 0.0) : cX;
+  const double cD = ex ? (partner_live ? cY : 0.0) : cX;
   // c_E' = cos c_E - s sin c_D ;  c_D' = cos c_D + s sin c_E  (no contraction)
   double nE, nD;
   if (!partner_live) {
@@ -168,8 +161,25 @@ __device__ __forceinline__ void forward_resolve(const TableT<KT>& t, const Facto
     nE = __dsub_rn(__dmul_rn(f.c, cE), __dmul_rn(ss, cD));
     nD = __dadd_rn(__dmul_rn(f.c, cD), __dmul_rn(ss, cE));
   }
-  const double nX = ex ? nE : nD;
-  const double nY = ex ? nD : nE;
+  nX = ex ? nE : nD;
+  nY = ex ? nD : nE;
+}
+
+// DEFER: created entries are appended unlinked (link_appended runs after the
+// step); otherwise they are hashed at once.
+template <bool RECORD, bool DEFER = false, class KT>
+__device__ __forceinline__ void forward_resolve(const TableT<KT>& t, const FactorT<KT>& f, int k, double eps,
+                                                unsigned int stamp, const TapeT<KT>& tape, unsigned long long i, KT X,
+                                                double cX, bool ex, const Lookup& r, StepCounts& sc) {
+  const KT Y = X ^ (f.occ | f.vir);
+  const bool partner_live = (r.state == ALIVE);
+  if (!ex && (partner_live || r.state == DEAD_NOW)) return;  // E's thread owns the pair
+  if (ex && r.state == DEAD_NOW) {
+    raise_consistency(t.cnt, SITE_PAIR_OWNER);
+    return;
+  }
+  double nX, nY;
+  rotate_member(f, X, cX, ex, partner_live, r.amp, nX, nY);
   ++sc.rot;
   if (t.entropy) {
     // Eq. 6 changes only on the pair: new terms (zero if dropped) minus old.
@@ -253,6 +263,34 @@ __device__ __forceinline__ void forward_entry(const TableT<KT>& t, const FactorT
   forward_resolve<RECORD>(t, f, k, eps, stamp, tape, i, X, cX, ex, r, sc);
 }
 
+// The reverse step of a pair with both members stored: (e0, d0) = U^T (e1, d1),
+// (lE, lD) = U^T (muE, muD), acc += s (lam_D psi_E - lam_E psi_D).  The reverse
+// sweep feeds only the gradient (no eps decision rests on it), so it contracts
+// to fused multiply-adds: fewer FP64 instructions, and each result rounded once.
+template <class KT>
+__device__ __forceinline__ void unrotate_pair(const FactorT<KT>& f, double ss, int parity, double e1, double d1,
+                                              double muE, double muD, double& e0, double& d0, double& lE, double& lD,
+                                              double& acc) {
+  e0 = fma(f.c, e1, ss * d1);
+  d0 = fma(f.c, d1, -(ss * e1));
+  lE = fma(f.c, muE, ss * muD);
+  lD = fma(f.c, muD, -(ss * muE));
+  acc = fma(neg_if(lD, parity), e0, acc);
+  acc = fma(neg_if(lE, parity ^ 1), d0, acc);
+}
+
+// The reverse step of a lone member X: its partner was absent before the
+// factor (and is not stored after it), so c_X' = cos c_X.  For X = E the
+// partner's adjoint is lam_D = -s mu_E and the term s lam_D psi_E; for X = D it
+// is lam_E = s mu_D and the term -s lam_E psi_D: both are -s (ss mu_X) psi_X.
+template <class KT>
+__device__ __forceinline__ void unrotate_lone(const FactorT<KT>& f, double ss, int parity, double cX, double muX,
+                                              double& x0, double& l0, double& acc) {
+  x0 = __dmul_rn(cX, f.ic);
+  acc = fma(neg_if(__dmul_rn(ss, muX), parity ^ 1), x0, acc);
+  l0 = __dmul_rn(f.c, muX);
+}
+
 // One stored entry i of the reverse step for factor k: psi_k -> psi_{k-1} in
 // place (inverse rotation on a stored pair, cos(theta) divided out of a lone
 // member), lambda_{k-1} = U_k^T mu_k, and this pair's share of
@@ -274,19 +312,8 @@ __device__ __forceinline__ void reverse_resolve(const TableT<KT>& t, const Facto
   const double ss = neg_if(f.s, parity);
   ++pairs;
   if (partner_live) {
-    // Both members stored: (e, d) = U^T (e', d'), (lamE, lamD) = U^T (muE, muD).
-    // The reverse sweep feeds only the gradient (no eps decision rests on
-    // it), so it contracts to fused multiply-adds: fewer FP64 instructions,
-    // and each result rounded once.
-    const double e1 = cX, d1 = r.amp;
-    const double muE = muX, muD = t.lam[r.idx];
-    const double e0 = fma(f.c, e1, ss * d1);
-    const double d0 = fma(f.c, d1, -(ss * e1));
-    const double lE = fma(f.c, muE, ss * muD);
-    const double lD = fma(f.c, muD, -(ss * muE));
-    // acc += s (lam_D psi_E - lam_E psi_D)
-    acc = fma(neg_if(lD, parity), e0, acc);
-    acc = fma(neg_if(lE, parity ^ 1), d0, acc);
+    double e0, d0, lE, lD;
+    unrotate_pair(f, ss, parity, cX, r.amp, muX, t.lam[r.idx], e0, d0, lE, lD, acc);
     if (t.born[i] == (unsigned int)k) {
       t.amps[i] = dead_value(stamp);
       ++kills;
@@ -302,14 +329,10 @@ __device__ __forceinline__ void reverse_resolve(const TableT<KT>& t, const Facto
       t.lam[r.idx] = lD;
     }
   } else {
-    // X alone: its partner was absent before the factor (and is not stored
-    // after it), so c_X' = cos c_X.  For X = E the partner's adjoint is
-    // lam_D = -s mu_E and the term s lam_D psi_E; for X = D it is
-    // lam_E = s mu_D and the term -s lam_E psi_D: both are -s (ss mu_X) psi_X.
-    const double x0 = __dmul_rn(cX, f.ic);
-    acc = fma(neg_if(__dmul_rn(ss, muX), parity ^ 1), x0, acc);
+    double x0, l0;
+    unrotate_lone(f, ss, parity, cX, muX, x0, l0, acc);
     t.amps[i] = x0;
-    t.lam[i] = __dmul_rn(f.c, muX);
+    t.lam[i] = l0;
   }
 }
 
