@@ -197,6 +197,11 @@ struct ucc_ctx {
   unsigned char* d_sb_rec = nullptr;
   size_t sb_rec_cap = 0;  // bytes
   RehashScratch rs;       // hash builds by regions
+  // Whole-grid resident passes: control words and inboxes (keys; two values per slot).
+  ResControl* d_res_ctl = nullptr;
+  unsigned long long* d_res_key = nullptr;
+  unsigned long long* d_res_val = nullptr;
+  size_t res_slots = 0;
   SelectState* d_sel = nullptr;
   void* d_cand = nullptr;  // SelectCandT<KT>[kSelectCandCap]: candidates of the cut's last selection passes
   double* d_entropy = nullptr;  // [K] Eq. 6 after each factor of the last apply
@@ -306,6 +311,7 @@ ucc_status check_device_error(const Counters& h) {
     msg += " consistency (site " + std::to_string(h.err_site) + ", key " + std::to_string(h.err_key) + ")";
   if (err & ERR_TAPE_FULL) msg += " tape-full";
   if (err & ERR_CAPACITY) msg += " capacity";
+  if (err & ERR_TIMEOUT) return fail(UCC_ETIMEOUT, msg + " a grid barrier timed out");
   return fail((err & (ERR_CAPACITY | ERR_TAPE_FULL)) ? UCC_ECAPACITY : UCC_ECUDA, msg);
 }
 
@@ -592,25 +598,50 @@ unsigned long long sector_bound(const ucc_ctx* c) {
   return d < 4.6e18 ? (unsigned long long)(d + 0.5) : 1ull << 62;
 }
 
-// Shape of the resident passes of a problem (k_resident.cu): for all its
-// tables where they fit a cluster's shared memory, else the largest shape,
-// for the factors at either end of a pass where the table is small.  False:
-// none, or options that speak of the launch-per-factor path (a fixed probe
-// width, an entry cap that its chunks check, the region-build test hook).
-bool resident_shape(const ucc_ctx* c, ResGeom* g, unsigned long long* bound) {
+// Determinants a problem's table can hold at a time: its sector, or twice
+// N_MAX (a factor at most doubles what the cut left).
+unsigned long long most_entries(const ucc_ctx* c) {
+  const unsigned long long sector = sector_bound(c);
+  return c->opt.n_max > 0 ? std::min(sector, 2ull * (unsigned long long)c->opt.n_max) : sector;
+}
+
+// Shape of the resident passes of a problem (k_resident.cu): a cluster where
+// it holds all its tables, else the whole grid, for as long as the table fits
+// it.  False: none, or options that speak of the launch-per-factor path (a
+// fixed probe width, an entry cap that its chunks check, the region-build
+// test hook).
+bool resident_shape(const ucc_ctx* c, ResGeom* g) {
   if (c->opt.rebuild_test_regions != 0 || c->opt.probe_width != 0 || c->opt.max_entries > 0) return false;
-  const int most = res_max_logC(c->kw);
-  if (most < 0) return false;
-  *bound = sector_bound(c);
-  unsigned long long need = *bound;
-  if (c->opt.n_max > 0) need = std::min(need, 2ull * (unsigned long long)c->opt.n_max);
-  *g = res_geometry(need, c->kw, most);
-  return true;
+  const ResLimits lim = res_limits(c->kw);
+  const unsigned long long most = most_entries(c);
+  return res_cluster_shape(most, c->kw, lim.cluster, g) || res_grid_shape(most, c->kw, lim.grid, g);
 }
 
 // Entries a table needs in global memory for what a resident pass can write back.
-unsigned long long resident_cap(const ResGeom& g, unsigned long long bound) {
-  return std::min<unsigned long long>((unsigned long long)g.L << g.logC, bound);
+unsigned long long resident_cap(const ucc_ctx* c, const ResGeom& g) {
+  return std::min<unsigned long long>((unsigned long long)g.L * (unsigned long long)g.ctas, sector_bound(c));
+}
+
+// Inboxes and control words of a whole-grid launch (kept by the context).
+template <class KT>
+ucc_status resident_net(ucc_ctx* c, const ResGeom& g, ResNet<KT>* net) {
+  *net = ResNet<KT>{};
+  if (!g.grid) return UCC_OK;
+  const size_t slots = 2ull * (size_t)g.ctas * (size_t)g.Lin;
+  if (!c->d_res_ctl) UCC_TRY(dalloc(&c->d_res_ctl, 1));
+  if (c->res_slots < slots) {
+    dfree(c->d_res_key);
+    dfree(c->d_res_val);
+    c->res_slots = 0;
+    UCC_TRY(dalloc(&c->d_res_key, slots * c->kw));
+    UCC_TRY(dalloc(&c->d_res_val, 2 * slots));
+    c->res_slots = slots;
+  }
+  net->ctl = c->d_res_ctl;
+  net->key = reinterpret_cast<KT*>(c->d_res_key);
+  net->a = reinterpret_cast<double*>(c->d_res_val);
+  net->b = c->d_res_val + c->res_slots;
+  return UCC_OK;
 }
 
 template <class KT>
@@ -669,8 +700,7 @@ ucc_status load_snapshot(ucc_ctx* c, TableSet& s, const Snapshot& snap) {
   unsigned long long cap = std::max<unsigned long long>(4 * snap.n, 1 << 12);
   {
     ResGeom g{};
-    unsigned long long bound = 0;
-    if (resident_shape(c, &g, &bound)) cap = std::max(cap, resident_cap(g, bound));
+    if (resident_shape(c, &g)) cap = std::max(cap, resident_cap(c, g));
   }
   if (cap >= kMaxEntries) return fail(UCC_ECAPACITY, "snapshot too large for one table");
   if (s.cur.cap_n < cap) UCC_TRY(s.cur.allocate(cap, slots_for(cap)));
@@ -806,7 +836,7 @@ ucc_status ensure_room(ucc_ctx* c, TableSet& s, bool record) {
 }
 
 template <class KT>
-ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, double eps, unsigned long long bound, int k0, int k1) {
+ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, const ResGeom& g, double eps, int k0, int k1) {
   ResJob<KT> j{};
   j.t = c->template table<KT>(s);
   j.factors = c->template dfactors<KT>();
@@ -815,16 +845,20 @@ ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, double eps, unsigne
   j.eps = eps;
   j.n_max = c->opt.n_max > 0 ? (unsigned long long)c->opt.n_max : 0ull;
   j.n_cut = c->opt.n_cut > 0 ? (unsigned long long)c->opt.n_cut : 0ull;
-  j.bound = bound;
+  j.bound = sector_bound(c);
+  j.most = std::min(most_entries(c), (unsigned long long)g.L * (unsigned long long)g.ctas);
   j.k0 = k0;
   j.k1 = k1;
   return j;
 }
 
-// More tape for a resident pass that holds h.tape_n records: twice as many
-// (few launches), or, past the call's budget, what the next factors need.
-ucc_status resident_tape(ucc_ctx* c, const Counters& h) {
-  const unsigned long long need = h.tape_n + 4ull * (h.n_tail - h.n_dead) + (1ull << 12);
+// Tape for a resident forward pass that holds h.tape_n records: room for the
+// records of a few full tables (the launch stops when half of that is left),
+// and twice what there is (few launches) unless that passes the call's budget.
+ucc_status resident_tape(ucc_ctx* c, const Counters& h, const ResGeom& g) {
+  const unsigned long long most =
+      std::min(most_entries(c), (unsigned long long)g.L * (unsigned long long)g.ctas);
+  const unsigned long long need = h.tape_n + 12ull * most + (1ull << 12);
   if (c->tape_cap >= need && c->tape_cap >= 2ull * h.tape_n) return UCC_OK;
   if (ensure_tape(c, std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
   c->tape_over_budget = false;
@@ -839,20 +873,21 @@ void resident_account(ucc_ctx* c, const Counters& h) {
   c->stats.peak_entries = std::max<long long>(c->stats.peak_entries, (long long)h.res_peak);
 }
 
-// As many of the factors [*k, k1) as one cluster can hold, on table s, whose
+// As many of the factors [*k, k1) as the shape holds, on table s, whose
 // counters the host mirror holds; *k moves to the first one left.
 template <class KT>
 ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, int* k, int k1) {
   ResGeom g{};
-  unsigned long long bound = 0;
-  if (!resident_shape(c, &g, &bound) || s.cur.cap_n < resident_cap(g, bound)) return UCC_OK;
+  if (!resident_shape(c, &g) || s.cur.cap_n < resident_cap(c, g)) return UCC_OK;
+  ResNet<KT> net{};
   while (*k < k1) {
-    const unsigned long long live = s.h_cnt->n_tail - s.h_cnt->n_dead;
-    if (!res_room_host(std::min(2ull * live, bound), g)) return UCC_OK;
-    if (record) UCC_TRY(resident_tape(c, *s.h_cnt));
-    CUDA_TRY(cudaMemsetAsync(&s.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
+    const Counters before = *s.h_cnt;
+    const unsigned long long live = before.n_tail - before.n_dead;
+    if (!res_room(live, g)) return UCC_OK;
+    UCC_TRY(resident_net<KT>(c, g, &net));
+    if (record) UCC_TRY(resident_tape(c, before, g));
     CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
-    CUDA_TRY(launch_res_forward<KT>(resident_job<KT>(c, s, eps, bound, *k, k1), nullptr, 1, g, record ? 1 : 0,
+    CUDA_TRY(launch_res_forward<KT>(resident_job<KT>(c, s, g, eps, *k, k1), nullptr, 1, g, net, record ? 1 : 0,
                                     c->stream));
     CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
     c->launches++;
@@ -862,7 +897,15 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
     CUDA_TRY(cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]));
     c->stats.forward_kernel_ms += ms;
     const Counters& h = *s.h_cnt;
-    if (h.res_status == RES_ABORT || h.res_k == *k) return UCC_OK;  // nothing was applied
+    if (h.res_status == RES_ABORT || h.res_k == *k) {  // nothing was applied
+      if (record && h.tape_n != before.tape_n) {
+        CUDA_TRY(cudaMemcpyAsync(&s.d_cnt->tape_n, &before.tape_n, sizeof(unsigned long long),
+                                 cudaMemcpyHostToDevice, c->stream));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        s.h_cnt->tape_n = before.tape_n;
+      }
+      return UCC_OK;
+    }
     if (h.res_k < *k || h.res_k > k1) return fail(UCC_ECUDA, "invalid resume factor");
     s.hash_valid = false;
     resident_account(c, h);
@@ -872,17 +915,18 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
   return UCC_OK;
 }
 
-// The reverse of the factors [k0, *k1) on table s as far as one cluster can
-// hold it; *k1 moves down to the first factor undone last.
+// The reverse of the factors [k0, k1) on table s in one resident launch, if it
+// fits; *done says so.
 template <class KT>
-ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int* k1) {
+ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int k1, bool* done) {
+  *done = false;
   ResGeom g{};
-  unsigned long long bound = 0;
-  if (!resident_shape(c, &g, &bound) || s.cur.cap_n < resident_cap(g, bound)) return UCC_OK;
-  if (!res_room_host(s.h_cnt->n_tail - s.h_cnt->n_dead, g)) return UCC_OK;
-  CUDA_TRY(cudaMemsetAsync(&s.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
+  if (!resident_shape(c, &g) || s.cur.cap_n < resident_cap(c, g)) return UCC_OK;
+  if (!res_room(s.h_cnt->n_tail - s.h_cnt->n_dead, g)) return UCC_OK;
+  ResNet<KT> net{};
+  UCC_TRY(resident_net<KT>(c, g, &net));
   CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
-  CUDA_TRY(launch_res_reverse<KT>(resident_job<KT>(c, s, 0.0, bound, k0, *k1), nullptr, 1, g, c->stream));
+  CUDA_TRY(launch_res_reverse<KT>(resident_job<KT>(c, s, g, 0.0, k0, k1), nullptr, 1, g, net, c->stream));
   CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
   c->launches++;
   c->stats.reverse_launches++;
@@ -892,15 +936,14 @@ ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int* k1) {
   c->stats.reverse_kernel_ms += ms;
   const Counters& h = *s.h_cnt;
   if (h.res_status == RES_ABORT) return UCC_OK;
-  if (h.res_k < k0 || h.res_k > *k1) return fail(UCC_ECUDA, "invalid resume factor");
   s.hash_valid = false;
   c->stats.reverse_compactions += (long long)h.res_rebuilds;
-  *k1 = h.res_k;
+  *done = true;
   return UCC_OK;
 }
 
-// Factors [k0, k1) on table s: resident in one cluster while the table is
-// small, then one launch per factor.  The last block of each factor flags a stop
+// Factors [k0, k1) on table s: resident while the table fits, then one launch
+// per factor.  The last block of each factor flags a stop
 // when the next factor might not fit or when the Methods-section cut is due;
 // later launches in the chunk then skip, and the host cuts / grows and
 // resumes at the flagged factor.  Chunks shrink when stops come often.
@@ -1031,9 +1074,8 @@ int segment_stride(const ucc_ctx* c) {
 template <class KT>
 ucc_status reset_for_run(ucc_ctx* c, TableSet& s) {
   ResGeom g{};
-  unsigned long long bound = 0;
-  const bool resident = c->K > 0 && resident_shape(c, &g, &bound);
-  return reset_table<KT>(c, s, !resident, resident ? resident_cap(g, bound) : 0ull);
+  const bool resident = c->K > 0 && resident_shape(c, &g);
+  return reset_table<KT>(c, s, !resident, resident ? resident_cap(c, g) : 0ull);
 }
 
 template <class KT>
@@ -1243,14 +1285,13 @@ ucc_status reverse_segment(ucc_ctx* c, TableSet& s, int k0, int k1) {
                            cudaMemcpyDeviceToHost, c->stream));
   UCC_TRY(read_counters(c, s));
   {
-    int k = k1;
-    UCC_TRY(resident_reverse<KT>(c, s, k0, &k));
-    if (k == k0) {
+    bool done = false;
+    UCC_TRY(resident_reverse<KT>(c, s, k0, k1, &done));
+    if (done) {
       c->stats.reverse_pairs += (long long)s.h_cnt->rev_pairs;
       c->stats.reverse_scanned += (long long)s.h_cnt->rev_scanned;
       return UCC_OK;
     }
-    k1 = k;
   }
   UCC_TRY(ensure_hash<KT>(c, s));
   const int grid_full = c->full_grid();
@@ -1496,6 +1537,9 @@ void destroy(ucc_ctx* c) {
   dfree(c->d_sb_fill);
   dfree(c->d_sb_off);
   dfree(c->d_sb_rec);
+  dfree(c->d_res_ctl);
+  dfree(c->d_res_key);
+  dfree(c->d_res_val);
   dfree(c->rs.rcnt);
   dfree(c->rs.rfill);
   dfree(c->rs.roff);
@@ -1582,10 +1626,7 @@ ucc_status run_alone(ucc_ctx* c, double eps, double* E, double* grad) {
 bool batch_resident_ok(const ucc_ctx* c, const ucc_options& first) {
   if (c->wide || c->K == 0 || first.batch_tiles != 0 || first.batch_test_skip_block != 0) return false;
   ResGeom g{};
-  unsigned long long bound = 0;
-  if (!resident_shape(c, &g, &bound)) return false;
-  if (c->opt.n_max > 0) bound = std::min(bound, 2ull * (unsigned long long)c->opt.n_max);
-  return res_fits(bound, 1, res_max_logC(1)) && c->opt.checkpoint_stride == 0 && c->opt.record_entropy == 0;
+  return resident_shape(c, &g) && !g.grid && c->opt.checkpoint_stride == 0 && c->opt.record_entropy == 0;
 }
 
 // The batched path for small tables: a cluster per job runs all its factors
@@ -1602,21 +1643,18 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
   for (int x : idx) record |= grads && grads[x];
   // The longest jobs first: they start first and the short ones fill in.
   std::vector<int> order(idx);
-  auto most_entries = [&](const ucc_ctx* c) {
-    const unsigned long long sector = sector_bound(c);
-    return c->opt.n_max > 0 ? std::min(sector, 2ull * (unsigned long long)c->opt.n_max) : sector;
-  };
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
     const ucc_ctx *x = jobs[a], *y = jobs[b];
     return (double)x->K * (4000.0 + (double)most_entries(x)) > (double)y->K * (4000.0 + (double)most_entries(y));
   });
-  unsigned long long bound = 1;
-  for (int x : order) bound = std::max(bound, most_entries(jobs[x]));
+  unsigned long long most = 1;
+  for (int x : order) most = std::max(most, most_entries(jobs[x]));
   // Clusters of eight keep twice as many jobs in flight as clusters of
   // sixteen, which pays from ten jobs on (nine large clusters fill the GPU).
-  int max_logC = res_max_logC(1);
-  if (n > 9 && max_logC > 3 && res_fits(bound, 1, 3)) max_logC = 3;
-  const ResGeom g = res_geometry(bound, 1, max_logC);
+  const int lim = res_limits(1).cluster;
+  ResGeom g{};
+  if (!(n > 9 && res_cluster_shape(most, 1, std::min(lim, 8), &g)) && !res_cluster_shape(most, 1, lim, &g))
+    return fail(UCC_ECUDA, "no cluster shape for a batch that has one");
   ResJob<KT>* d_jobs = nullptr;
   JobView* d_view = nullptr;
   JobState* d_js = nullptr;
@@ -1644,9 +1682,12 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
       c->have_entropy = false;
       c->have_psi = c->have_sigma = false;
       UCC_TRY(settle_spare(c, c->ts[0]));
-      UCC_TRY(reset_table<KT>(c, c->ts[0], false, resident_cap(g, sector_bound(c))));
-      if (record) UCC_TRY(reset_tape(c, c->ts[0], 0));
+      UCC_TRY(reset_table<KT>(c, c->ts[0], false, resident_cap(c, g)));
       *c->ts[0].h_cnt = Counters{};
+      if (record) {
+        UCC_TRY(reset_tape(c, c->ts[0], 0));
+        UCC_TRY(resident_tape(c, *c->ts[0].h_cnt, g));
+      }
     }
     // Counters of the jobs in `which`, one synchronisation for all.
     auto read_all = [&](const std::vector<int>& which) -> ucc_status {
@@ -1662,7 +1703,8 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
     auto upload = [&](const std::vector<int>& which, bool reverse) -> ucc_status {
       for (size_t y = 0; y < which.size(); ++y) {
         ucc_ctx* c = jobs[which[y]];
-        hj[y] = resident_job<KT>(c, c->ts[0], eps, sector_bound(c), reverse ? 0 : c->ts[0].h_cnt->res_k, c->K);
+        const int k0 = reverse ? 0 : c->ts[0].h_cnt->res_k;
+        hj[y] = resident_job<KT>(c, c->ts[0], g, eps, k0, c->K);
       }
       CUDA_TRY(cudaMemcpyAsync(d_jobs, hj.data(), which.size() * sizeof(ResJob<KT>), cudaMemcpyHostToDevice, st));
       return UCC_OK;
@@ -1672,7 +1714,7 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
     std::vector<int> todo(order), done;
     while (!todo.empty()) {
       UCC_TRY(upload(todo, false));
-      CUDA_TRY(launch_res_forward<KT>(hj[0], d_jobs, (int)todo.size(), g, record ? 1 : 0, st));
+      CUDA_TRY(launch_res_forward<KT>(hj[0], d_jobs, (int)todo.size(), g, ResNet<KT>{}, record ? 1 : 0, st));
       UCC_TRY(read_all(todo));
       std::vector<int> more;
       for (int x : todo) {
@@ -1686,7 +1728,7 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
           done.push_back(x);
         } else if (h.res_status == RES_TAPE) {
           resident_account(c, h);
-          UCC_TRY(resident_tape(c, h));
+          UCC_TRY(resident_tape(c, h, g));
           more.push_back(x);
         } else {
           alone->push_back(x);
@@ -1733,7 +1775,7 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
       CUDA_TRY(launch_lambda_init_batch(d_view, d_js, m, d_bh, c0->full_grid(), st));
       UCC_TRY(upload(jobs_in, true));
       CUDA_TRY(cudaEventRecord(c0->ev[4], st));
-      CUDA_TRY(launch_res_reverse<KT>(hj[0], d_jobs, m, g, st));
+      CUDA_TRY(launch_res_reverse<KT>(hj[0], d_jobs, m, g, ResNet<KT>{}, st));
       CUDA_TRY(cudaEventRecord(c0->ev[5], st));
     }
     CUDA_TRY(cudaMemcpyAsync(hs.data(), d_js, m * sizeof(JobState), cudaMemcpyDeviceToHost, st));

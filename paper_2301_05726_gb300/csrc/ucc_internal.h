@@ -62,14 +62,14 @@ struct Counters {
   // Result of the last resident launch (ResStatus; next factor; its cuts,
   // rebuilds and largest entry count).
   int res_status, res_k;
-  unsigned long long res_cut;
+  unsigned long long res_cut, res_n;  // res_n: entries written back (0 between launches)
   unsigned int res_rebuilds, res_peak;
 };
 
 // How a resident launch ended.
 enum ResStatus : int {
   RES_DONE = 1,   // every factor asked for
-  RES_FULL = 2,   // before factor res_k (forward) or below it (reverse): the next one might not fit
+  RES_FULL = 2,   // forward, before factor res_k: it might not fit
   RES_TAPE = 3,   // forward, before factor res_k: more kill tape is needed
   RES_ABORT = 4   // a CTA's share outgrew its arrays: nothing was written back
 };
@@ -92,7 +92,8 @@ enum DeviceError : int {
   ERR_PROBE_BOUND = 1,   // a probe ran past its step bound (table too full)
   ERR_CONSISTENCY = 2,   // a state the algorithm excludes was observed
   ERR_TAPE_FULL = 4,     // kill tape capacity exceeded
-  ERR_CAPACITY = 8       // entry allocation past capacity
+  ERR_CAPACITY = 8,      // entry allocation past capacity
+  ERR_TIMEOUT = 16       // a resident launch's grid barrier gave up waiting
 };
 
 // Everything a kernel needs to address the wavefunction table.
@@ -163,14 +164,15 @@ struct __align__(32) SigRecT {
 };
 static_assert(sizeof(SigRecT<unsigned long long>) == 32, "record is one sector");
 
-// Shape of a resident launch (k_resident.cu): 2^logC CTAs a cluster, each with
-// room for L entries and 2^logB hash buckets of four slots.
+// Shape of a resident launch (k_resident.cu): CTAs that share a table (a
+// thread-block cluster, or the whole grid), each with room for L entries, Lin
+// messages and 2^logB hash buckets of four slots.
 struct ResGeom {
-  int logC, L, logB;
+  int ctas, grid, L, Lin, logB;
 };
 
 // One job of a resident launch: factors [k0, k1) of a table that holds at most
-// `bound` determinants (its sector).
+// `bound` determinants (its sector), and at most `most` at a time here.
 template <class KT>
 struct ResJob {
   TableT<KT> t;
@@ -178,8 +180,34 @@ struct ResJob {
   TapeT<KT> tape;
   double* grad;
   double eps;
-  unsigned long long n_max, n_cut, bound;  // the cut (n_max 0: none)
+  unsigned long long n_max, n_cut, bound, most;  // the cut (n_max 0: none)
   int k0, k1;
+};
+
+// Control words of a resident launch over the whole grid, cleared before it:
+// the barrier's ring, messages received [buffer][kind][CTA] (a sector each),
+// and the cut's histogram and candidates.
+struct ResControl {
+  unsigned long long words[4][16];
+  unsigned int count[2][2][240][8];
+  unsigned int hist[4096];
+  unsigned int ncand, pad[3];
+  unsigned long long cand_mag[512], cand_key[1024];
+};
+
+// ... and its inboxes, [2][ctas][Lin] each (null for clusters).
+template <class KT>
+struct ResNet {
+  ResControl* ctl;
+  KT* key;
+  double* a;
+  unsigned long long* b;
+};
+
+// Largest cluster, and CTAs of a whole-grid launch, that the current device
+// runs the resident kernels with (0: none).
+struct ResLimits {
+  int cluster, grid;
 };
 
 // Radix-selection state of the N_MAX / N_CUT truncation.
@@ -372,21 +400,21 @@ cudaError_t launch_persist_reverse(JobView* jobs, JobState* js, int n_jobs, Batc
                                    int tiles, cudaStream_t st);
 // The persistent kernels' grid (blocks resident at once) on the current device.
 int persist_grid(int record, int probe_width, int reverse);
-// Resident passes: a cluster per job runs all its factors in shared memory.
-// res_geometry: the shape for tables of at most `bound` entries (clusters of at
-// most 2^max_logC CTAs); res_fits: whether any shape holds them.  many (n_jobs
-// of them, device memory) or, when null, the single job `one`.
-ResGeom res_geometry(unsigned long long bound, int key_words, int max_logC);
-bool res_fits(unsigned long long bound, int key_words, int max_logC);
-bool res_room_host(unsigned long long bound, const ResGeom& g);  // ... whether shape g does
-// Largest cluster (log2 of its CTAs) the current device runs these kernels in; -1: none.
-int res_max_logC(int key_words);
+// Resident passes: one launch runs a run of factors with the table in shared
+// memory.  res_cluster_shape: a cluster for tables of at most `most` entries
+// (false: too large); res_grid_shape: the whole grid, sized for them as far as
+// it goes; res_room: whether a shape holds that many.
+ResLimits res_limits(int key_words);
+bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, ResGeom* g);
+bool res_grid_shape(unsigned long long most, int key_words, int ctas, ResGeom* g);
+bool res_room(unsigned long long entries, const ResGeom& g);
+// many: n_jobs jobs in device memory, or null for the single job `one`.
 template <class KT>
 cudaError_t launch_res_forward(const ResJob<KT>& one, const ResJob<KT>* many, int n_jobs, const ResGeom& g,
-                               int record, cudaStream_t st);
+                               const ResNet<KT>& net, int record, cudaStream_t st);
 template <class KT>
 cudaError_t launch_res_reverse(const ResJob<KT>& one, const ResJob<KT>* many, int n_jobs, const ResGeom& g,
-                               cudaStream_t st);
+                               const ResNet<KT>& net, cudaStream_t st);
 // Message returned by ucc_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

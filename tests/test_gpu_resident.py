@@ -1,13 +1,14 @@
-"""Resident passes (a whole run of factors in one thread-block cluster, the
-table in its shared memory) against the launch-per-factor kernels and the CPU
-oracle: the same determinants and bit-identical amplitudes, counts, entropies
+"""Resident passes (a whole run of factors in one launch, the table in the
+shared memory of a thread-block cluster or of the whole GPU) against the
+launch-per-factor kernels and the CPU oracle: the same determinants and bit-identical amplitudes, counts, entropies
 (1e-10), energies (1e-10 Ha) and gradients (1e-8).
 
 The shapes sit where the resident kernels change behaviour: every cluster size,
 tables below and above one thread per entry, heavy eps drops with revivals,
 cuts that keep one entry or all but a few, ties larger than the ranked
-candidate list (also on the key's words), two-word keys, a table that outgrows
-the cluster on the way, and a tape that needs more than one launch.
+candidate list (also on the key's words), two-word keys, tables just above the
+clusters' size and of the whole GPU's, a table that outgrows the GPU's shared
+memory on the way, and a tape that needs more than one launch.
 """
 import numpy as np
 import pytest
@@ -54,12 +55,18 @@ def problem(name):
         "ties": lambda: make(9, 4, 4, cut=(5000, 4001), pre=260, zero_from=8),
         "ties_wide": lambda: make(36, 3, 3, cut=(3000, 2501), pre=200, zero_from=8),
         "wide_eps_cut": lambda: make(40, 4, 3, eps=1e-6, cut=(1601, 1000), pre=250),
-        "outgrows": lambda: make(12, 4, 4, pre=260),
+        "grid": lambda: make(12, 4, 4, pre=260),
+        "grid_drops_and_revivals": lambda: make(11, 4, 3, eps=1e-4, sigma=0.2, pre=400),
+        "grid_cut": lambda: make(14, 4, 4, eps=1e-9, cut=(30001, 17001), pre=220),
+        "grid_ties": lambda: make(12, 4, 4, cut=(20000, 16001), pre=220, zero_from=8),
+        "grid_ties_wide": lambda: make(36, 3, 3, cut=(20000, 16001), pre=330, zero_from=8),
+        "grid_wide": lambda: make(34, 3, 3, eps=1e-7, cut=(24000, 15000), pre=260),
     }[name]()
 
 
 CASES = ["one_cta", "one_cta_open_shell_eps", "four_ctas", "eight_ctas", "sixteen_ctas", "drops_and_revivals",
-         "cut_keeps_all", "cut_keeps_one", "cut_odd", "ties", "ties_wide", "wide_eps_cut", "outgrows"]
+         "cut_keeps_all", "cut_keeps_one", "cut_odd", "ties", "ties_wide", "wide_eps_cut", "grid",
+         "grid_drops_and_revivals", "grid_cut", "grid_ties", "grid_ties_wide", "grid_wide"]
 
 
 def same_state(got, want):
@@ -81,10 +88,7 @@ def test_state_and_gradient(torch_cuda, name):
     same_state(ctx.wavefunction(), (ok, oa))
     for c in ("rotations", "created", "dropped_new", "dropped_old", "cut"):
         assert st[c] == oc[c], c
-    if name != "outgrows":
-        assert st["forward_launches"] == 1  # the resident path ran
-    else:
-        assert st["forward_launches"] > 1  # resident to begin with, then a launch per factor
+    assert st["forward_launches"] == 1  # the resident path ran
     E, g = ctx.gradient()
     assert abs(E - E_o) <= E_TOL and np.max(np.abs(g - g_o)) <= G_TOL
     general = UCCContext(p)
@@ -96,7 +100,7 @@ def test_state_and_gradient(torch_cuda, name):
     assert abs(E - Eg) <= E_TOL and np.max(np.abs(g - gg)) <= G_TOL
 
 
-@pytest.mark.parametrize("name", ["one_cta_open_shell_eps", "sixteen_ctas", "cut_odd", "outgrows"])
+@pytest.mark.parametrize("name", ["one_cta_open_shell_eps", "sixteen_ctas", "cut_odd", "grid_cut"])
 def test_entropy(torch_cuda, name):
     import oracle
     from paper_2301_05726_gb300.api import UCCContext
@@ -108,13 +112,32 @@ def test_entropy(torch_cuda, name):
     assert np.max(np.abs(ctx.entropy() - S)) <= 1e-10
 
 
-@pytest.mark.parametrize("stride", [1, 37])
-def test_segments(torch_cuda, stride):
+def test_outgrows_the_gpu(torch_cuda):
+    # Resident to begin with; past some 700,000 determinants a launch per factor.
+    from paper_2301_05726_gb300.api import UCCContext
+    p = synth.make_problem(77, 15, 4, 4, 0.08).prefix(900)
+    ctx, general = UCCContext(p), UCCContext(p)
+    general.set_options(rebuild_test_regions=1)
+    for c in (ctx, general):
+        c.apply()
+    st, sg = ctx.stats(), general.stats()
+    assert 1 < st["forward_launches"] < sg["forward_launches"] and st["n_det"] > 900_000
+    for c in ("n_det", "rotations", "created"):
+        assert st[c] == sg[c], c
+    same_state(ctx.wavefunction(), general.wavefunction())
+    E, g = ctx.gradient()
+    Eg, gg = general.gradient()
+    assert abs(E - Eg) <= E_TOL and np.max(np.abs(g - gg)) <= G_TOL
+
+
+@pytest.mark.parametrize("name,pre,stride", [("cut_odd", 150, 1), ("cut_odd", 150, 37), ("grid_cut", 120, 11)])
+def test_segments(torch_cuda, name, pre, stride):
     # Checkpointed gradients run each segment resident, forward and reverse.
     import oracle
     from paper_2301_05726_gb300.api import UCCContext
-    p = problem("cut_odd").prefix(150)
-    p.n_max, p.n_cut = 2999, 1701
+    whole = problem(name)
+    p = whole.prefix(pre)
+    p.n_max, p.n_cut = whole.n_max, whole.n_cut
     ctx = UCCContext(p)
     ctx.set_options(checkpoint_stride=stride)
     E, g = ctx.gradient()
@@ -144,7 +167,7 @@ def test_batch_mixes_cluster_sizes_and_paths(torch_cuda):
     # Jobs of every size share a launch; a job too large for a cluster and a
     # two-word one take their own paths in the same call.
     from paper_2301_05726_gb300.api import UCCContext, batch_run
-    names = ["one_cta", "cut_odd", "eight_ctas", "outgrows", "ties", "wide_eps_cut", "cut_keeps_one", "four_ctas",
+    names = ["one_cta", "cut_odd", "eight_ctas", "grid", "ties", "wide_eps_cut", "cut_keeps_one", "four_ctas",
              "sixteen_ctas", "drops_and_revivals", "one_cta_open_shell_eps", "cut_keeps_all"]
     probs = [problem(n) for n in names]
     ctxs = [UCCContext(p) for p in probs]
