@@ -183,8 +183,9 @@ struct ucc_ctx {
   ucc_options opt{};
 
   void* d_factors = nullptr;     // FactorT<KT>[K]
-  double* d_h = nullptr;
-  double* d_g = nullptr;
+  double* d_h = nullptr;         // [n^2], then (same allocation)
+  double* d_g = nullptr;         // [n^4]
+  double* d_fock = nullptr;      // [2 n^3 + (n (n - 1) / 2)^2] tables of the bucketed energy (launch_fock_tables)
   double* d_grad = nullptr;
   double* d_partials = nullptr;
   int partial_cap = 0;
@@ -357,7 +358,7 @@ ucc_status ensure_rehash_scratch(ucc_ctx* c, unsigned long long cap, unsigned lo
     r.regions = 0;
     UCC_TRY(dalloc(&r.rcnt, regions));
     UCC_TRY(dalloc(&r.rfill, regions));
-    UCC_TRY(dalloc(&r.roff, regions + 1));
+    UCC_TRY(dalloc(&r.roff, sb_offsets(regions)));
     r.regions = regions;
   }
   if (!r.over_n) UCC_TRY(dalloc(&r.over_n, 1));
@@ -1132,17 +1133,23 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
   const Counters h = *s.h_cnt;
   const unsigned long long n = h.n_tail, live = h.n_tail - h.n_dead;
   const unsigned long long ne = (unsigned long long)(c->n_alpha + c->n_beta);
-  const unsigned long long est = live * (ne + ne * (ne - 1) / 2);
+  const unsigned long long est_d = live * (ne * (ne - 1) / 2), est_s = live * ne;
+  const unsigned long long est = est_d + est_s;  // the records, exactly
   if (est == 0) {
     if (must) return fail(UCC_ESTATE, "no stored determinant to bucket");
     return UCC_OK;
   }
-  int log2p = 0;
-  if (c->opt.energy_test_partitions > 0)
-    while ((1 << log2p) < c->opt.energy_test_partitions) ++log2p;
-  else
-    while (log2p < 24 && (est >> log2p) > (unsigned long long)sb_partition_target()) ++log2p;
-  const unsigned long long P = 1ull << log2p;
+  SbParts pt{0, 0};
+  auto grow = [&](unsigned long long records, int* log2p) {
+    while (*log2p < 24 && (records >> *log2p) > (unsigned long long)sb_partition_target(c->kw)) ++*log2p;
+  };
+  if (c->opt.energy_test_partitions > 0) {
+    while ((1 << pt.log2d) < c->opt.energy_test_partitions) ++pt.log2d;
+  } else {
+    grow(est_d, &pt.log2d);
+    grow(est_s, &pt.log2s);
+  }
+  const unsigned long long P = (1ull << pt.log2d) + (1ull << pt.log2s);
   auto unavailable = [&](const char* what) -> ucc_status {
     if (must) return fail(UCC_ENOMEM, std::string("bucketed energy: ") + what);
     cudaGetLastError();  // clear a failed allocation
@@ -1154,7 +1161,7 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
     dfree(c->d_sb_off);
     c->sb_parts = 0;
     if (dalloc(&c->d_sb_cnt, P) != UCC_OK || dalloc(&c->d_sb_fill, P) != UCC_OK ||
-        dalloc(&c->d_sb_off, P + 1) != UCC_OK) {
+        dalloc(&c->d_sb_off, sb_offsets(P)) != UCC_OK) {
       dfree(c->d_sb_cnt);
       dfree(c->d_sb_fill);
       dfree(c->d_sb_off);
@@ -1163,9 +1170,9 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
     c->sb_parts = P;
   }
   const size_t rec_bytes = sb_record_bytes(c->wide ? 2 : 1);
-  size_t free_b = 0, total_b = 0;
-  CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
   const size_t want = std::min<size_t>(kSbBudgetBytes, (size_t)est * rec_bytes);
+  size_t free_b = 0, total_b = 0;
+  if (c->sb_rec_cap < want) CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
   if (c->sb_rec_cap < want && c->sb_rec_cap < (size_t)(kSbBudgetShare * (double)(free_b + c->sb_rec_cap))) {
     dfree(c->d_sb_rec);
     c->sb_rec_cap = 0;
@@ -1184,31 +1191,31 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
   SigRecT<KT>* rec = reinterpret_cast<SigRecT<KT>*>(c->d_sb_rec);
   CUDA_TRY(cudaMemsetAsync(c->d_sb_cnt, 0, P * sizeof(unsigned int), c->stream));
   CUDA_TRY(cudaMemsetAsync(t.sigma, 0, n * sizeof(double), c->stream));
-  CUDA_TRY(launch_sb_count(t, c->d_sb_cnt, log2p, grid, c->stream));
+  CUDA_TRY(launch_sb_count(t, c->d_sb_cnt, pt, grid, c->stream));
   CUDA_TRY(launch_sb_scan(c->d_sb_cnt, c->d_sb_off, P, c->stream));
-  c->launches += 2;
+  c->launches += 3;
   auto off_at = [&](unsigned long long p, unsigned long long* v) -> ucc_status {
     CUDA_TRY(cudaMemcpyAsync(v, c->d_sb_off + p, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     return UCC_OK;
   };
-  unsigned long long total = 0;
-  UCC_TRY(off_at(P, &total));
-  *records = total;
-  // Rounds: partition ranges whose records fit the buffer, halved until they do.
+  *records = est;
+  // Rounds: partition ranges whose records fit the buffer, halved until they
+  // do.  Where all fit, nothing needs to be read back.
+  const bool one_round = est <= cap_recs;
   std::vector<std::pair<unsigned long long, unsigned long long>> todo;
   {
-    const unsigned long long rounds = std::max<unsigned long long>(1ull, (total + cap_recs - 1) / cap_recs);
-    unsigned long long width = P;
-    while (width > 1 && P / width < rounds) width >>= 1;
-    for (unsigned long long p = P; p > 0; p -= width) todo.push_back({p - width, p});
+    const unsigned long long rounds = std::min(P, std::max<unsigned long long>(1ull, (est + cap_recs - 1) / cap_recs));
+    for (unsigned long long x = rounds; x-- > 0;) todo.push_back({P * x / rounds, P * (x + 1) / rounds});
   }
   while (!todo.empty()) {
     const auto [p0, p1] = todo.back();
     todo.pop_back();
-    unsigned long long a = 0, b = 0;
-    UCC_TRY(off_at(p0, &a));
-    UCC_TRY(off_at(p1, &b));
+    unsigned long long a = 0, b = est;
+    if (!one_round) {
+      UCC_TRY(off_at(p0, &a));
+      UCC_TRY(off_at(p1, &b));
+    }
     if (b - a > cap_recs) {
       if (p1 - p0 == 1) return fail(UCC_ECAPACITY, "one core partition outgrew the record buffer");
       const unsigned long long mid = p0 + (p1 - p0) / 2;
@@ -1218,10 +1225,9 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
     }
     if (b == a) continue;
     CUDA_TRY(cudaMemsetAsync(c->d_sb_fill + p0, 0, (p1 - p0) * sizeof(unsigned int), c->stream));
-    CUDA_TRY(launch_sb_scatter(t, c->d_sb_off, c->d_sb_fill, rec, log2p, p0, p1, a, grid, c->stream));
-    CUDA_TRY(launch_sb_pairs(t, in, rec, c->d_sb_off, log2p, p0, p1, a,
-                             (int)std::min<unsigned long long>((unsigned long long)pair_grid, p1 - p0), c->stream));
-    c->launches += 2;
+    CUDA_TRY(launch_sb_scatter(t, c->d_sb_off, c->d_sb_fill, rec, pt, p0, p1, a, grid, c->stream));
+    CUDA_TRY(launch_sb_pairs(t, in, rec, c->d_sb_off, pt, p0, p1, a, pair_grid, c->stream));
+    c->launches += 3;
   }
   CUDA_TRY(launch_sb_finish(t, in, grid, c->stream));
   c->launches++;
@@ -1237,6 +1243,9 @@ ucc_status run_energy(ucc_ctx* c, double* E, double* norm2) {
   in.g = c->d_g;
   in.n = c->n_spatial;
   in.n_so = c->n_so;
+  in.fsame = c->d_fock;
+  in.fother = c->d_fock + (size_t)c->n_spatial * c->n_spatial * c->n_spatial;
+  in.anti = in.fother + (size_t)c->n_spatial * c->n_spatial * c->n_spatial;
   UCC_TRY(read_counters(c, s));
   const unsigned long long n = s.h_cnt->n_tail;
   int grid = (int)std::min<unsigned long long>((unsigned long long)c->full_grid(), (n + 7) / 8);
@@ -1530,7 +1539,6 @@ void destroy(ucc_ctx* c) {
   for (auto& sn : c->snaps) sn.release();
   dfree(c->d_factors);
   dfree(c->d_h);
-  dfree(c->d_g);
   dfree(c->d_grad);
   dfree(c->d_partials);
   dfree(c->d_sb_cnt);
@@ -2207,8 +2215,11 @@ ucc_status ucc_create(const ucc_hamiltonian* ham, const ucc_ansatz* an, void* cu
   c->d_factors = fb;
   if ((s = dalloc(&cb, cbytes * kSelectCandCap)) != UCC_OK) return bail(s);
   c->d_cand = cb;
-  if ((s = dalloc(&c->d_h, n * n)) != UCC_OK) return bail(s);
-  if ((s = dalloc(&c->d_g, n * n * n * n)) != UCC_OK) return bail(s);
+  // h, g and the bucketed energy's tables: one allocation
+  if ((s = dalloc(&c->d_h, n * n + n * n * n * n + 2 * n * n * n + n * (n - 1) / 2 * (n * (n - 1) / 2))) != UCC_OK)
+    return bail(s);
+  c->d_g = c->d_h + n * n;
+  c->d_fock = c->d_g + n * n * n * n;
   if ((s = dalloc(&c->d_grad, std::max(1, c->K))) != UCC_OK) return bail(s);
   if ((s = c->ts[0].init()) != UCC_OK) return bail(s);
   if ((s = c->ts[1].init()) != UCC_OK) return bail(s);
@@ -2225,6 +2236,15 @@ ucc_status ucc_create(const ucc_hamiltonian* ham, const ucc_ansatz* an, void* cu
       cudaMemcpyAsync(c->d_g, ham->g, n * n * n * n * sizeof(double), cudaMemcpyHostToDevice, c->stream) !=
           cudaSuccess)
     return bail(fail(UCC_ECUDA, "integral upload failed"));
+  {
+    Integrals in;
+    in.h = c->d_h;
+    in.g = c->d_g;
+    in.n = c->n_spatial;
+    in.n_so = c->n_so;
+    if (launch_fock_tables(in, c->d_fock, c->d_fock + n * n * n, c->d_fock + 2 * n * n * n, c->stream) != cudaSuccess)
+      return bail(fail(UCC_ECUDA, "integral tables failed"));
+  }
   if ((s = upload_factors(c)) != UCC_OK) return bail(s);
   *out = c;
   return UCC_OK;

@@ -147,6 +147,15 @@ struct Integrals {
   const double* g;  // [n^4] chemist (pq|rs)
   int n;            // spatial orbitals
   int n_so;
+  const double* fsame = nullptr;   // [n^3] (pr|kk) - (pk|kr) at (p n + r) n + k (bucketed energy)
+  const double* fother = nullptr;  // [n^3] (pr|kk)
+  const double* anti = nullptr;    // [(n (n - 1) / 2)^2] (ar|bs) - (as|br), pairs a < b, r < s
+};
+
+// Partitions of the bucketed energy: 2^log2d for the doubles' cores, then 2^log2s
+// for the singles'.
+struct SbParts {
+  int log2d, log2s;
 };
 
 // One record of the bucketed energy: a core K (a stored determinant with one
@@ -316,6 +325,10 @@ cudaError_t launch_compact(const TableT<KT>& from, const TableT<KT>& to, int wit
 template <class KT>
 cudaError_t launch_rehash(const TableT<KT>& t, int grid, cudaStream_t st);
 
+// launch_sb_scan's result for n counts: n + 1 offsets and the sums of its tiles.
+constexpr unsigned long long kSbScanTile = 4096;
+constexpr unsigned long long sb_offsets(unsigned long long n) { return n + 1 + (n + kSbScanTile - 1) / kSbScanTile; }
+
 // Scratch of the hash build by regions (one-word keys): per region of
 // 2^kRegionBits slots its entry count, fill counter and offset, the (key,
 // index) pairs bucketed by region, and the pairs whose probe runs past their
@@ -324,7 +337,7 @@ constexpr int kRegionBits = 13;
 struct RehashScratch {
   unsigned int* rcnt = nullptr;         // [regions]
   unsigned int* rfill = nullptr;        // [regions]
-  unsigned long long* roff = nullptr;   // [regions + 1]
+  unsigned long long* roff = nullptr;   // [sb_offsets(regions)]
   unsigned long long* pairs = nullptr;  // [2 * cap]
   unsigned long long* over = nullptr;   // [2 * cap]
   unsigned long long* over_n = nullptr; // [1]
@@ -351,21 +364,23 @@ cudaError_t launch_lambda_init(const TableT<KT>& t, int grid, cudaStream_t st);
 // of partitions [p0, p1) (fill: per-partition counters, zeroed per round),
 // the pair sums into sigma, and the diagonal with E and <psi|psi>.
 template <class KT>
-cudaError_t launch_sb_count(const TableT<KT>& t, unsigned int* cnt, int log2p, int grid, cudaStream_t st);
+cudaError_t launch_sb_count(const TableT<KT>& t, unsigned int* cnt, SbParts pt, int grid, cudaStream_t st);
 cudaError_t launch_sb_scan(const unsigned int* cnt, unsigned long long* off, unsigned long long n, cudaStream_t st);
 template <class KT>
 cudaError_t launch_sb_scatter(const TableT<KT>& t, const unsigned long long* off, unsigned int* fill,
-                              SigRecT<KT>* rec, int log2p, unsigned long long p0, unsigned long long p1,
+                              SigRecT<KT>* rec, SbParts pt, unsigned long long p0, unsigned long long p1,
                               unsigned long long base, int grid, cudaStream_t st);
 template <class KT>
 cudaError_t launch_sb_pairs(const TableT<KT>& t, const Integrals& in, const SigRecT<KT>* rec,
-                            const unsigned long long* off, int log2p, unsigned long long p0, unsigned long long p1,
+                            const unsigned long long* off, SbParts pt, unsigned long long p0, unsigned long long p1,
                             unsigned long long base, int grid, cudaStream_t st);
 template <class KT>
 cudaError_t launch_sb_finish(const TableT<KT>& t, const Integrals& in, int grid, cudaStream_t st);
+// The bucketed energy's tables of a problem (Integrals::fsame, fother, anti).
+cudaError_t launch_fock_tables(const Integrals& in, double* fsame, double* fother, double* anti, cudaStream_t st);
 size_t sb_record_bytes(int key_words);
 int sb_blocks_per_sm(int key_words);
-int sb_partition_target();  // mean records per partition the host aims for
+int sb_partition_target(int key_words);  // mean records per partition the host aims for
 // rs (may be null): scratch of a hash build by regions, used to hash a bulk
 // re-insertion's appended range into a large one-word table.
 template <class KT>
