@@ -143,26 +143,21 @@ __global__ void __launch_bounds__(kThreads) k_link_tail(TableT<KT> t) {
 template <class KT, int G>
 __global__ void __launch_bounds__(kStepThreads, 8) k_reverse(TableT<KT> t, const FactorT<KT>* __restrict__ factors,
                                                              int k, unsigned int stamp, double* grad) {
-  // The adjoint of a linked entry is prefetched into L2 when the entry is
-  // queued and loaded with its partner's filter word (staging it with every
-  // scanned entry costs more than it saves).
-  __shared__ LinkScratch<KT> s_w[kStepThreads / 32];
+  __shared__ ReverseScratchT<KT> s_w[kStepThreads / 32];
   const FactorT<KT> f = factors[k];
   const unsigned long long n = min(*((volatile unsigned long long*)&t.cnt->n_tail), t.cap_n);
-  double acc = 0.0;
-  unsigned int pairs = 0, kills = 0;
-  for_each_linked<false>(
-      t, f, n, s_w[threadIdx.x >> 5], nullptr, [&](unsigned long long i, bool act) { return act ? t.lam[i] : 0.0; },
-      [&](unsigned long long i, KT X, double cX, bool ex, double mu, bool act) {
-        if (act) reverse_resolve(t, f, k, stamp, i, X, cX, mu, ex, absent_lookup(), acc, pairs, kills);
-      },
-      [&](unsigned long long i, KT X, double cX, bool ex, double, bool act) {
+  double acc = 0.0, lone = 0.0;
+  unsigned int pairs = 0, kills = 0, settled = 0;
+  scan_reverse(
+      t, f, (unsigned int)n, s_w[threadIdx.x >> 5],
+      [&](unsigned long long i, KT X, double cX, bool ex, bool act) {
         const double mu = act ? t.lam[i] : 0.0;
-        Lookup r = findG<G>(t, X ^ (f.occ | f.vir), act, stamp);
+        const Lookup r = findG<G>(t, X ^ (f.occ | f.vir), act, stamp);
         if (act) reverse_resolve(t, f, k, stamp, i, X, cX, mu, ex, r, acc, pairs, kills);
       },
-      // the adjoint of a queued entry moves towards L2 while the scan goes on
-      [&](unsigned long long i) { prefetch_l2(&t.lam[i]); });
+      lone, settled);
+  acc = fma(-f.s, lone, acc);
+  if ((threadIdx.x & 31u) == 0u) pairs += settled;
   {
     // Entries this step removed (born at factor k) count as dropped, so the
     // host can compact the table when they pile up.

@@ -47,11 +47,12 @@ __device__ __forceinline__ void block_add_counts(Counters* c, unsigned long long
 // this step carry this step's stamp, so a D-thread can tell "E was live when
 // the step began" (live or DEAD_NOW) from "E absent" (ABSENT or DEAD_OLD).
 template <class KT, int G, bool RECORD>
-__global__ void __launch_bounds__(kStepThreads, 8) k_forward(TableT<KT> t, const FactorT<KT>* __restrict__ factors,
+__global__ void __launch_bounds__(kStepThreads, 6) k_forward(TableT<KT> t, const FactorT<KT>* __restrict__ factors,
                                                              int k, double eps, unsigned int stamp, TapeT<KT> tape,
                                                              unsigned long long n_max) {
   __shared__ int s_skip;
-  __shared__ LinkScratch<KT> s_w[kStepThreads / 32];
+  __shared__ ForwardScratchT<KT> s_w[kStepThreads / 32];
+  __shared__ CreateQueueT<KT> s_made[kStepThreads / 32];
   if (threadIdx.x == 0) s_skip = *((volatile int*)&t.cnt->stop_k) >= 0;
   __syncthreads();
   // An earlier factor of this chunk stopped it: every block of the launch
@@ -62,15 +63,29 @@ __global__ void __launch_bounds__(kStepThreads, 8) k_forward(TableT<KT> t, const
   {
     const FactorT<KT> f = factors[k];
     const unsigned long long n = min(*((volatile unsigned long long*)&t.cnt->n_scan), t.cap_n);
-    for_each_linked<false>(
-        t, f, n, s_w[threadIdx.x >> 5], nullptr, [](unsigned long long, bool) { return 0.0; },
-        [&](unsigned long long i, KT X, double cX, bool ex, double, bool act) {
-          if (act) forward_resolve<RECORD, true>(t, f, k, eps, stamp, tape, i, X, cX, ex, absent_lookup(), sc);
+    CreateQueueT<KT>& made = s_made[threadIdx.x >> 5];
+    int n_made = 0;         // warp-uniform
+    unsigned int sure = 0;  // entries settled by the scan (warp-uniform)
+    scan_forward(
+        t, f, (unsigned int)n, eps, t.entropy == nullptr, s_w[threadIdx.x >> 5],
+        [&](unsigned long long i, KT X, double cX, bool ex, bool act) {
+          double c = 0.0;
+          const bool add =
+              act && forward_resolve<RECORD, true>(t, f, k, eps, stamp, tape, i, X, cX, ex, absent_lookup(), sc, &c);
+          queue_created(t, made, n_made, add, X ^ (f.occ | f.vir), c, (unsigned int)k, RECORD);
         },
-        [&](unsigned long long i, KT X, double cX, bool ex, double, bool act) {
-          Lookup r = findG<G>(t, X ^ (f.occ | f.vir), act, stamp);
-          if (act) forward_resolve<RECORD, true>(t, f, k, eps, stamp, tape, i, X, cX, ex, r, sc);
-        });
+        [&](unsigned long long i, KT X, double cX, bool ex, bool act) {
+          const Lookup r = findG<G>(t, X ^ (f.occ | f.vir), act, stamp);
+          double c = 0.0;
+          const bool add = act && forward_resolve<RECORD, true>(t, f, k, eps, stamp, tape, i, X, cX, ex, r, sc, &c);
+          queue_created(t, made, n_made, add, X ^ (f.occ | f.vir), c, (unsigned int)k, RECORD);
+        },
+        sure);
+    if ((threadIdx.x & 31u) == 0u) {  // a rotation each, its partner dropped at once
+      sc.rot += sure;
+      sc.dnew += sure;
+    }
+    if (n_made > 0) flush_created(t, made, n_made, n_made, (unsigned int)k, RECORD);
   }
   block_add_counts(t.cnt, sc.rot, sc.cre, sc.dnew, sc.dold, sc.dead_delta);
   if (t.entropy) {
@@ -571,17 +586,18 @@ namespace {
 // G-lane probes (the autotuner times it); the result only feeds a checksum.
 template <class KT, int G>
 __global__ void __launch_bounds__(kStepThreads) k_probe_bench(TableT<KT> t, FactorT<KT> f, unsigned long long* sink) {
-  __shared__ LinkScratch<KT> s_w[kStepThreads / 32];
+  __shared__ ForwardScratchT<KT> s_w[kStepThreads / 32];
   const unsigned long long n = min(*((volatile unsigned long long*)&t.cnt->n_tail), t.cap_n);
   const KT m = f.occ | f.vir;
   unsigned long long acc = 0;
-  for_each_linked<false>(
-      t, f, n, s_w[threadIdx.x >> 5], nullptr, [](unsigned long long, bool) { return 0.0; },
-      [&](unsigned long long, KT, double, bool, double, bool) {},
-      [&](unsigned long long, KT X, double, bool, double, bool act) {
-        Lookup r = findG<G>(t, X ^ m, act, 0u);
+  unsigned int sure = 0;
+  scan_forward(
+      t, f, (unsigned int)n, 0.0, false, s_w[threadIdx.x >> 5], [](unsigned long long, KT, double, bool, bool) {},
+      [&](unsigned long long, KT X, double, bool, bool act) {
+        const Lookup r = findG<G>(t, X ^ m, act, 0u);
         if (act) acc += r.idx + (unsigned long long)r.state;
-      });
+      },
+      sure);
   acc = warp_sum_u64(acc);
   if ((threadIdx.x & 31u) == 0 && acc) atomicAdd(sink, acc);
 }

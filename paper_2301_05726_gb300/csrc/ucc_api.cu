@@ -791,7 +791,8 @@ ucc_status autotune(ucc_ctx* c, TableSet& s, int k, unsigned long long n) {
       }
       float ms = 0.f;
       cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]);
-      if (rep == 1 && (w == 1 || ms < best_ms)) {
+      // (a wider probe must be clearly faster: the replay is short)
+      if (rep == 1 && (w == 1 || ms < 0.9f * best_ms)) {
         best_ms = ms;
         best = w;
       }
@@ -1359,8 +1360,11 @@ ucc_status reverse_segment(ucc_ctx* c, TableSet& s, int k0, int k1) {
       CUDA_TRY(launch_tape_reinsert(c->template table<KT>(s), c->template tape<KT>(), k, rec, std::max(g2, 1),
                                     c->stream, &c->launches, by_regions ? &c->rs : nullptr, c->num_sms));
     }
+    // One lane per probe unless the width is fixed: the sweep's probes are few
+    // and mostly hits in the home slot, and a wider one takes its queries in
+    // turn (64 spin-orbitals, all steps: 283, 290, 317 and 377 ms for 1, 2, 4 and 8).
     CUDA_TRY(launch_reverse(c->template table<KT>(s), c->template dfactors<KT>(), k, stamp, c->d_grad,
-                            pick_probe_width(c), grid, c->stream));
+                            c->opt.probe_width > 0 ? c->opt.probe_width : 1, grid, c->stream));
     c->launches++;
     c->stats.reverse_launches++;
     bound += rec;

@@ -78,21 +78,57 @@ __device__ __forceinline__ void record_kill(const TableT<KT>& t, const TapeT<KT>
 // lanes); in_range is false for lanes past the end of the table.
 // The rotation, creation and eps rule for one linked entry i (key X, live
 // amplitude cX, ex = X is the excited member) whose partner lookup is r.
-// Append a created entry without hashing it: within a factor step no thread
-// looks a created key up (its only partner is the creating entry), so the
-// slot is claimed after the step (link_appended) and the claim's round trip
-// stays off the step's critical path.
+// Entries a factor step creates, gathered per warp in shared memory and
+// appended 32 at a time without a hash slot: within a step no thread looks a
+// created key up (its only partner is the creating entry), so the slot is
+// claimed after the step (link_appended).  Most drains of 32 linked entries
+// create one or two; an append each made 1e5 additions to the table's
+// one tail counter per factor, which the step waited for: k_forward and k_link
+// over 2,184 factors at 64 spin-orbitals and 1e7 determinants 215 and, batched, 184 ms.
+constexpr int kCreateQueue = 64;
 template <class KT>
-__device__ __forceinline__ void append_unlinked(const TableT<KT>& t, KT key, double amp, unsigned int born,
-                                                bool with_born) {
-  const unsigned long long idx = aggregated_add(&t.cnt->n_tail);
-  if (idx >= t.cap_n) {
-    raise_error(t.cnt, ERR_CAPACITY);
-    return;
+struct CreateQueueT {
+  KT X[kCreateQueue];
+  double c[kCreateQueue];
+};
+
+// Append the last `take` (<= 32) of the n queued entries.  All lanes call this.
+template <class KT>
+__device__ __forceinline__ void flush_created(const TableT<KT>& t, CreateQueueT<KT>& q, int& n, int take,
+                                              unsigned int born, bool with_born) {
+  const int lane = (int)(threadIdx.x & 31u);
+  unsigned long long base = 0ull;
+  if (lane == 0) base = atomicAdd(&t.cnt->n_tail, (unsigned long long)take);
+  base = __shfl_sync(0xFFFFFFFFu, base, 0);
+  __syncwarp();  // the queue's last writes
+  n -= take;
+  if (lane < take) {
+    const unsigned long long idx = base + (unsigned long long)lane;
+    if (idx < t.cap_n) {
+      t.keys[idx] = q.X[n + lane];
+      t.amps[idx] = q.c[n + lane];
+      if (with_born) t.born[idx] = born;
+    } else {
+      raise_error(t.cnt, ERR_CAPACITY);
+    }
   }
-  t.keys[idx] = key;
-  t.amps[idx] = amp;
-  if (with_born) t.born[idx] = born;
+  __syncwarp();  // read before the slots are reused
+}
+
+// Queue the lanes' created entries (made); flushes full batches.  All lanes
+// call this; n is warp-uniform.
+template <class KT>
+__device__ __forceinline__ void queue_created(const TableT<KT>& t, CreateQueueT<KT>& q, int& n, bool made, KT X,
+                                              double c, unsigned int born, bool with_born) {
+  const unsigned int m = __ballot_sync(0xFFFFFFFFu, made);
+  if (m == 0u) return;
+  if (made) {
+    const int p = n + __popc(m & ((1u << (threadIdx.x & 31u)) - 1u));
+    q.X[p] = X;
+    q.c[p] = c;
+  }
+  n += __popc(m);
+  if (n >= 32) flush_created(t, q, n, 32, born, with_born);
 }
 
 // Give appended entry idx its hash slot unless its key already has one (a
@@ -165,18 +201,20 @@ __device__ __forceinline__ void rotate_member(const FactorT<KT>& f, KT X, double
   nY = ex ? nD : nE;
 }
 
-// DEFER: created entries are appended unlinked (link_appended runs after the
-// step); otherwise they are hashed at once.
+// DEFER: a created partner's amplitude is returned in *made with true (the
+// caller appends it: queue_created); otherwise it is appended and hashed at
+// once and the result is false.
 template <bool RECORD, bool DEFER = false, class KT>
-__device__ __forceinline__ void forward_resolve(const TableT<KT>& t, const FactorT<KT>& f, int k, double eps,
+__device__ __forceinline__ bool forward_resolve(const TableT<KT>& t, const FactorT<KT>& f, int k, double eps,
                                                 unsigned int stamp, const TapeT<KT>& tape, unsigned long long i, KT X,
-                                                double cX, bool ex, const Lookup& r, StepCounts& sc) {
+                                                double cX, bool ex, const Lookup& r, StepCounts& sc,
+                                                double* made = nullptr) {
   const KT Y = X ^ (f.occ | f.vir);
   const bool partner_live = (r.state == ALIVE);
-  if (!ex && (partner_live || r.state == DEAD_NOW)) return;  // E's thread owns the pair
+  if (!ex && (partner_live || r.state == DEAD_NOW)) return false;  // E's thread owns the pair
   if (ex && r.state == DEAD_NOW) {
     raise_consistency(t.cnt, SITE_PAIR_OWNER);
-    return;
+    return false;
   }
   double nX, nY;
   rotate_member(f, X, cX, ex, partner_live, r.amp, nX, nY);
@@ -224,12 +262,14 @@ __device__ __forceinline__ void forward_resolve(const TableT<KT>& t, const Facto
     }
     ++sc.cre;
   } else {
-    if (DEFER)
-      append_unlinked(t, Y, nY, (unsigned int)k, RECORD);
-    else
-      insert_new(t, Y, nY, (unsigned int)k, r.slot, RECORD, false, SITE_CREATE_DUP);
     ++sc.cre;
+    if (DEFER) {
+      *made = nY;
+      return true;
+    }
+    insert_new(t, Y, nY, (unsigned int)k, r.slot, RECORD, false, SITE_CREATE_DUP);
   }
+  return false;
 }
 
 // Scan half of a factor step: whether stored entry i (in_range false past the
@@ -356,54 +396,38 @@ __device__ __forceinline__ void reverse_entry(const TableT<KT>& t, const FactorT
 // FP64 pipe, where a warp instruction costs the same with one lane as with 32)
 // and the partner probes on mostly idle lanes, and every lane would wait for
 // the slowest lane's probe chain.  Instead the lanes append the linked entries
-// they find to a queue; each 32 taken from it test their partners' filter
-// bits together, the lanes whose partner is proved absent resolve at once
-// (no slot probe), and the rest move to a probe queue that is resolved, slot
-// probe first, 32 at a time.  The order in which a step's pairs are resolved
-// does not matter: ownership and the dropped-entry stamps decide everything
-// from the state at the start of the step.
+// that need more than their own values to queues and resolve them 32 at a time.
+// The order in which a step's pairs are resolved does not matter: ownership and
+// the dropped-entry stamps decide everything from the state at the start of the
+// step.
 //
-// The keys and amplitudes of a warp's next round of kScanTiles tiles (and,
-// with AUX, a third per-entry array: the adjoint in the reverse sweep) are
-// copied into shared memory (cp.async, two buffers per warp) while it works on
+// The keys and amplitudes of the warp's coming rounds of kScanTiles tiles are
+// copied into shared memory (cp.async, three buffers per warp) while it works on
 // the current one, so the scan's load latency overlaps the pair work and a
 // linked entry's own values never need a load of their own.
 constexpr int kScanTiles = 2;
 constexpr int kRound = 32 * kScanTiles;
-constexpr int kQueue = 64;
+constexpr int kQueue = 32 + kRound;  // a round's entries on top of a partial batch
 // Queue entries keep the entry index in 31 bits and the excited-member flag in
 // the top bit: the host keeps every table below kMaxEntries entries.
 constexpr unsigned int kExBit = 1u << 31;
 static_assert(kMaxEntries <= (1ull << 31), "queue indices are 31-bit");
 
-template <class KT, bool AUX>
+template <class KT>
 struct LinkQueueT {
   unsigned int i[kQueue];  // entry index, kExBit set for the excited member
   KT X[kQueue];
   double c[kQueue];
-  double m[AUX ? kQueue : 1];
 };
 
-template <class KT, bool AUX>
+template <class KT>
 struct __align__(16) ScanStageT {
   KT X[kRound];
   double c[kRound];
-  double m[AUX ? kRound : 2];
 };
 
-// Per-warp shared memory of for_each_linked.
-template <class KT, bool AUX>
-struct LinkScratchT {
-  ScanStageT<KT, AUX> stage[2];
-  LinkQueueT<KT, AUX> linked;  // linked entries, before the filter test
-  LinkQueueT<KT, AUX> probe;   // linked entries whose partner may be stored
-};
-template <class KT>
-using LinkScratch = LinkScratchT<KT, false>;
-
-// Threads per block of the kernels built on for_each_linked: with four warps
-// per block, the eight blocks an SM holds at 64 registers per thread also fit
-// its shared memory with their LinkScratch.
+// Threads per block of the scanning kernels: with four warps per block, six to
+// eight blocks an SM fit its registers and its shared memory.
 constexpr int kStepThreads = 128;
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int src_bytes) {
@@ -421,29 +445,28 @@ inline bool scan_aligned(const TableT<KT>& t) {
            reinterpret_cast<uintptr_t>(t.lam)) & 15u) == 0u;
 }
 
-// Copy entries [base, min(base + kRound, n)) of keys and amps (and aux) into a
-// stage: 16-byte pieces of two entries (of one entry for two-word keys); the
-// piece holding entry n - 1 alone copies 8 bytes (the rest zero-filled) and
-// pieces past n are not issued.
-template <class KT, bool AUX>
-__device__ __forceinline__ void stage_round(const TableT<KT>& t, const double* aux, ScanStageT<KT, AUX>& st,
-                                            unsigned long long base, unsigned long long n, unsigned int lane) {
+// Copy entries [base, min(base + kRound, n)) of keys and amps into a stage:
+// 16-byte pieces of two entries (of one entry for two-word keys); the piece
+// holding entry n - 1 alone copies 8 bytes (the rest zero-filled) and pieces past
+// n are not issued.
+template <class KT>
+__device__ __forceinline__ void stage_round(const TableT<KT>& t, ScanStageT<KT>& st, unsigned int base,
+                                            unsigned int n, unsigned int lane) {
 #pragma unroll
   for (int h = 0; h < kRound / 64; ++h) {
     const int e = 2 * (int)(lane + 32u * h);  // first entry of the piece, relative to base
-    const unsigned long long g = base + (unsigned long long)e;
+    const unsigned int g = base + (unsigned int)e;
     if (g < n) {
-      const int bytes = g + 1ull < n ? 16 : 8;
+      const int bytes = g + 1 < n ? 16 : 8;
       if (sizeof(KT) == 8) cp_async16(&st.X[e], t.keys + g, bytes);
       cp_async16(&st.c[e], t.amps + g, bytes);
-      if (AUX) cp_async16(&st.m[e], aux + g, bytes);
     }
   }
   if (sizeof(KT) == 16) {
 #pragma unroll
     for (int h = 0; h < kRound / 32; ++h) {
       const int e = (int)(lane + 32u * h);
-      const unsigned long long g = base + (unsigned long long)e;
+      const unsigned int g = base + (unsigned int)e;
       if (g < n) cp_async16(&st.X[e], t.keys + g, 16);
     }
   }
@@ -459,142 +482,277 @@ __device__ __forceinline__ Lookup absent_lookup() {
   return r;
 }
 
-// Append (i, X, c, ex, m) of the active lanes (ballot mk) to queue q at qn.
-template <class KT, bool AUX>
-__device__ __forceinline__ void enqueue(LinkQueueT<KT, AUX>& q, int qn, unsigned int mk, unsigned int below_me,
-                                        bool act, unsigned long long i, KT X, double c, bool ex, double m) {
+// Append (i, X, c, ex) of the active lanes (ballot mk) to queue q at qn.
+template <class KT>
+__device__ __forceinline__ void enqueue(LinkQueueT<KT>& q, int qn, unsigned int mk, unsigned int below_me, bool act,
+                                        unsigned int i, KT X, double c, bool ex) {
   if (act) {
     const int p = qn + __popc(mk & below_me);
-    q.i[p] = (unsigned int)i | (ex ? kExBit : 0u);
+    q.i[p] = i | (ex ? kExBit : 0u);
     q.X[p] = X;
     q.c[p] = c;
-    if (AUX) q.m[p] = m;
   }
 }
 
 // Pop the last 32 entries of a queue holding qn >= 32 into the lanes and call
-// f(i, X, c, ex, m, true).
-template <class KT, bool AUX, class F>
-__device__ __forceinline__ void drain32(LinkQueueT<KT, AUX>& q, int& qn, unsigned int lane, F& f) {
+// f(i, X, c, ex, true).
+template <class KT, class F>
+__device__ __forceinline__ void drain32(LinkQueueT<KT>& q, int& qn, unsigned int lane, F& f) {
   __syncwarp();
   const int p = qn - 32 + (int)lane;
   const unsigned int qi = q.i[p];
   const KT qX = q.X[p];
   const double qc = q.c[p];
-  const double qm = AUX ? q.m[p] : 0.0;
   __syncwarp();
   qn -= 32;
-  f((unsigned long long)(qi & ~kExBit), qX, qc, (qi & kExBit) != 0u, qm, true);
+  f((unsigned long long)(qi & ~kExBit), qX, qc, (qi & kExBit) != 0u, true);
 }
 
 // The qn < 32 entries left in a queue (lanes past qn inactive); empties it.
-template <class KT, bool AUX, class F>
-__device__ __forceinline__ void drain_rest(LinkQueueT<KT, AUX>& q, int& qn, unsigned int lane, F& f) {
+template <class KT, class F>
+__device__ __forceinline__ void drain_rest(LinkQueueT<KT>& q, int& qn, unsigned int lane, F& f) {
   __syncwarp();
   const bool a = (int)lane < qn;
   unsigned int qi = 0u;
   KT qX = KeyOps<KT>::zero();
-  double qc = 0.0, qm = 0.0;
+  double qc = 0.0;
   if (a) {
     qi = q.i[lane];
     qX = q.X[lane];
     qc = q.c[lane];
-    if (AUX) qm = q.m[lane];
   }
   __syncwarp();
   qn = 0;
-  f((unsigned long long)(qi & ~kExBit), qX, qc, (qi & kExBit) != 0u, qm, a);
+  f((unsigned long long)(qi & ~kExBit), qX, qc, (qi & kExBit) != 0u, a);
 }
 
-// Scan entries [0, n) in warp-strided rounds of kRound entries and resolve
-// every live linked entry: lone(i, X, cX, ex, m, active) when the filter
-// proves its partner absent, probe(i, X, cX, ex, m, active) otherwise, where m
-// is the entry's value in aux (AUX: staged with the scan) or, without AUX,
-// pre(i, active) for lone entries (loaded together with the filter word, so a
-// lone entry waits for a single round trip) and 0 for probed ones.  Every lane
-// of the warp calls this; lone and probe are called by all lanes together.
-// hint(i) is called for each live linked entry i when it is queued (a
-// prefetch of what its resolution will load).
-template <bool AUX, class KT, class Pre, class Lone, class Probe, class Hint>
-__device__ __forceinline__ void for_each_linked(const TableT<KT>& t, const FactorT<KT>& f, unsigned long long n,
-                                                LinkScratchT<KT, AUX>& w, const double* aux, Pre pre, Lone lone,
-                                                Probe probe, Hint hint) {
+// Largest exponent field of an amplitude cX for which |s cX| is certainly below
+// eps, rounding included: |cX| < 2^(e + 1 - 1023), so the product stays below
+// 2^(e + es + 2 - 2046), and one exponent more of room keeps its rounded value below
+// eps >= 2^(e_eps - 1023).  -1: none (eps zero or subnormal).
+__device__ __forceinline__ int surely_below(double s, double eps) {
+  const int es = (__double2hiint(s) >> 20) & 0x7FF, ee = (__double2hiint(eps) >> 20) & 0x7FF;
+  return ee == 0 ? -1 : min(ee + 1020 - es, 0x7FE);
+}
+
+// Per-warp shared memory of scan_forward: three rounds of keys and amplitudes
+// and the two queues.
+template <class KT>
+struct ForwardScratchT {
+  ScanStageT<KT> stage[3];
+  LinkQueueT<KT> lone, probe;
+};
+
+// The forward step's scan.  At 64 spin-orbitals 95 % of the linked entries have
+// an absent partner whose new amplitude falls below eps, which the exponents
+// nearly always tell: such an entry is only multiplied by cos(theta).  It is
+// settled where it is scanned -- filter word, one product, its own eps test, a
+// store -- without its sign, the partner's amplitude or a queue (counted in
+// `sure`, per warp).  The others are queued and resolved 32 at a time: lone(i, X,
+// cX, ex, active) when the filter proved the partner absent, probe(the same)
+// otherwise, both called by all lanes together.  settle: false sends every entry
+// through the queues.
+// Settling took a step from 65 to 40 million warp instructions, and then the
+// filter words' round trip was what it waited for; so the words of round r + 1
+// are loaded before round r is worked on, while round r + 2 is copied in
+// (k_forward and k_link over the 2,184
+// factors of that problem: 184 ms with the queues alone, 168 ms so).
+template <class KT, class Lone, class Probe>
+__device__ __forceinline__ void scan_forward(const TableT<KT>& t, const FactorT<KT>& f, unsigned int n,
+                                             double eps, bool settle, ForwardScratchT<KT>& w, Lone lone, Probe probe,
+                                             unsigned int& sure) {
   const unsigned int lane = threadIdx.x & 31u;
   const unsigned int below_me = (1u << lane) - 1u;
-  const unsigned long long warp = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  const unsigned long long step = nwarps * (unsigned long long)kRound;
+  const unsigned int step = ((gridDim.x * blockDim.x) >> 5) * (unsigned int)kRound;  // (n + 3 step < 2^32)
   const KT m = f.occ | f.vir;
-  int nl = 0, np = 0;  // warp-uniform lengths of the linked and probe queues
-  // Up to 32 linked entries: the partner's filter bit sends each lane to lone
-  // at once or onto the probe queue.
-  auto split = [&](unsigned long long i, KT X, double c, bool ex, double mu, bool act) {
-    if (!AUX) mu = pre(i, act);
-    bool maybe = act;
-    if (act && t.filt) {
-      const unsigned long long h = KeyOps<KT>::filt_hash(X ^ m);
-      maybe = filter_hit(t, t.filt[filter_word(t, h)], h);
-    }
-    const bool pr = act && maybe;
-    const unsigned int mp = __ballot_sync(0xFFFFFFFFu, pr);
-    enqueue<KT, AUX>(w.probe, np, mp, below_me, pr, i, X, c, ex, mu);
-    np += __popc(mp);
-    lone(i, X, c, ex, mu, act && !maybe);
-    if (np >= 32) drain32<KT, AUX>(w.probe, np, lane, probe);
-  };
-  unsigned long long base = warp * (unsigned long long)kRound;
-  if (base < n) stage_round<KT, AUX>(t, aux, w.stage[0], base, n, lane);
-  cp_async_commit();
-  for (int r = 0; base < n; base += step, ++r) {
-    // Next round's copy into the other buffer (its last reader was round r - 1).
-    if (base + step < n) stage_round<KT, AUX>(t, aux, w.stage[(r + 1) & 1], base + step, n, lane);
+  const int lim = settle ? surely_below(f.s, eps) : -1;
+  int nl = 0, np = 0;  // warp-uniform lengths of the lone and probe queues
+  auto stage = [&](int b, unsigned int at) {
+    if (at < n) stage_round(t, w.stage[b], at, n, lane);
     cp_async_commit();
-    cp_async_wait_all_but_last();  // this round's copy has landed (this lane's pieces)
-    __syncwarp();                  // ... and every other lane's
-    const ScanStageT<KT, AUX>& st = w.stage[r & 1];
-    // Not unrolled: the body inlines the resolve paths (instruction cache).
-#pragma unroll 1
+  };
+  // A tile's lookups on their way: the filter word, the key's bits in it (0:
+  // not linked, or past the end -- the stage then holds stale entries), and
+  // whether the entry is the excited member.
+  unsigned int word[kScanTiles], bits[kScanTiles];
+  bool ex[kScanTiles];
+  auto look = [&](int b, unsigned int at) {
+    const ScanStageT<KT>& st = w.stage[b];
+#pragma unroll
     for (int u = 0; u < kScanTiles; ++u) {
       const int e = 32 * u + (int)lane;
-      const unsigned long long i = base + (unsigned long long)e;
-      bool act = false, ex = false;
-      KT X = KeyOps<KT>::zero();
-      double cX = 0.0, mu = 0.0;
-      if (i < n) {
-        X = st.X[e];
-        // occ and vir are disjoint: E holds exactly occ of the factor's
-        // orbitals, D exactly vir
-        const KT tX = X & m;
-        ex = tX == f.occ;
-        if (ex || tX == f.vir) {
-          cX = st.c[e];
-          act = !is_dead(cX);
-          if (AUX) mu = st.m[e];
-        }
+      const KT X = st.X[e];
+      // occ and vir are disjoint: E holds exactly occ of the factor's orbitals, D
+      // exactly vir.
+      const KT tX = X & m;
+      ex[u] = tX == f.occ;
+      const bool act = (ex[u] || tX == f.vir) && at + (unsigned int)e < n && !is_dead(st.c[e]);
+      word[u] = 0xFFFFFFFFu;
+      bits[u] = 0u;
+      if (act) {
+        const unsigned long long h = KeyOps<KT>::filt_hash(X ^ m);
+        bits[u] = filter_bits(t, h);
+        if (t.filt) word[u] = t.filt[filter_word(t, h)];
       }
-      const unsigned int ml = __ballot_sync(0xFFFFFFFFu, act);
-      if (act) hint(i);
-      enqueue<KT, AUX>(w.linked, nl, ml, below_me, act, i, X, cX, ex, mu);
-      nl += __popc(ml);
-      if (nl >= 32) drain32<KT, AUX>(w.linked, nl, lane, split);
     }
+  };
+  unsigned int base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (unsigned int)kRound;
+  stage(0, base);
+  stage(1, base + step);
+  cp_async_wait_all_but_last();
+  __syncwarp();
+  if (base < n) look(0, base);
+  for (int b = 0; base < n; base += step, b = b == 2 ? 0 : b + 1) {
+    const int b1 = b == 2 ? 0 : b + 1, b2 = b1 == 2 ? 0 : b1 + 1;
+    // (buffer b2's last reader was the round before this one)
+    stage(b2, base + 2 * step);
+    cp_async_wait_all_but_last();  // the next round's copy has landed (this lane's pieces)
+    __syncwarp();                  // ... and every other lane's
+    unsigned int wd[kScanTiles], fb[kScanTiles];
+    bool e0[kScanTiles];
+#pragma unroll
+    for (int u = 0; u < kScanTiles; ++u) {
+      wd[u] = word[u];
+      fb[u] = bits[u];
+      e0[u] = ex[u];
+    }
+    if (base + step < n) look(b1, base + step);
+    const ScanStageT<KT>& st = w.stage[b];
+#pragma unroll
+    for (int u = 0; u < kScanTiles; ++u) {
+      const int x = 32 * u + (int)lane;
+      const unsigned int i = base + (unsigned int)x;
+      const bool act = fb[u] != 0u, absent = (wd[u] & fb[u]) != fb[u];
+      const double c = st.c[x];
+      bool done = act && absent && ((__double2hiint(c) >> 20) & 0x7FF) <= lim;
+      if (done) {
+        const double p = __dmul_rn(f.c, c);
+        done = !below_eps(p, eps);
+        if (done) t.amps[i] = p;
+      }
+      sure += __popc(__ballot_sync(0xFFFFFFFFu, done));
+      const bool q = act && !done;
+      const unsigned int mq = __ballot_sync(0xFFFFFFFFu, q);
+      if (mq) {
+        const unsigned int ml = __ballot_sync(0xFFFFFFFFu, q && absent), mp = mq & ~ml;
+        enqueue(w.lone, nl, ml, below_me, q && absent, i, st.X[x], c, e0[u]);
+        enqueue(w.probe, np, mp, below_me, q && !absent, i, st.X[x], c, e0[u]);
+        nl += __popc(ml);
+        np += __popc(mp);
+      }
+    }
+#pragma unroll 1
+    while (nl >= 32) drain32(w.lone, nl, lane, lone);
+#pragma unroll 1
+    while (np >= 32) drain32(w.probe, np, lane, probe);
     __syncwarp();  // every lane is done with this buffer before it is refilled
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");  // nothing left in flight
-  if (nl > 0) drain_rest<KT, AUX>(w.linked, nl, lane, split);
-  if (np > 0) drain_rest<KT, AUX>(w.probe, np, lane, probe);
+  if (nl > 0) drain_rest(w.lone, nl, lane, lone);
+  if (np > 0) drain_rest(w.probe, np, lane, probe);
 }
 
-template <bool AUX, class KT, class Pre, class Lone, class Probe>
-__device__ __forceinline__ void for_each_linked(const TableT<KT>& t, const FactorT<KT>& f, unsigned long long n,
-                                                LinkScratchT<KT, AUX>& w, const double* aux, Pre pre, Lone lone,
-                                                Probe probe) {
-  for_each_linked<AUX>(t, f, n, w, aux, pre, lone, probe, [](unsigned long long) {});
-}
+// Per-warp shared memory of scan_reverse.
+template <class KT>
+struct ReverseScratchT {
+  ScanStageT<KT> stage[3];
+  LinkQueueT<KT> probe;
+};
 
-// Bring the line holding p into L2 (no register result, no wait).
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+// The reverse step's scan, built like scan_forward, with the adjoint loaded
+// beside the filter word, a round ahead.  An entry whose partner the filter
+// proves absent is alone: its amplitude over cos(theta), its adjoint times it, and
+// their product added to `lone` (the sign of a lone member's term of the gradient
+// is the same for E and D: unrotate_lone's, summed without its -sin(theta)).  The
+// other linked entries are queued for probe(i, X, cX, ex, active).  pairs counts
+// the lone ones, per warp.  A quarter of the scanned entries is alone, so the
+// three FP64 products run on a quarter of the lanes and that pipe is 55 % busy
+// (DRAM 57 %); gathering lone entries 32 at a time first was measured and is
+// slower (k_reverse and re-insertion at 64 spin-orbitals 359 against 283 ms).
+template <class KT, class Probe>
+__device__ __forceinline__ void scan_reverse(const TableT<KT>& t, const FactorT<KT>& f, unsigned int n,
+                                             ReverseScratchT<KT>& w, Probe probe, double& lone,
+                                             unsigned int& pairs) {
+  const unsigned int lane = threadIdx.x & 31u;
+  const unsigned int below_me = (1u << lane) - 1u;
+  const unsigned int step = ((gridDim.x * blockDim.x) >> 5) * (unsigned int)kRound;  // (n + 3 step < 2^32)
+  const KT m = f.occ | f.vir;
+  int np = 0;  // warp-uniform length of the probe queue
+  auto stage = [&](int b, unsigned int at) {
+    if (at < n) stage_round(t, w.stage[b], at, n, lane);
+    cp_async_commit();
+  };
+  unsigned int word[kScanTiles], bits[kScanTiles];  // as in scan_forward
+  bool ex[kScanTiles];
+  double mu[kScanTiles];
+  auto look = [&](int b, unsigned int at) {
+    const ScanStageT<KT>& st = w.stage[b];
+#pragma unroll
+    for (int u = 0; u < kScanTiles; ++u) {
+      const int e = 32 * u + (int)lane;
+      const KT X = st.X[e];
+      const KT tX = X & m;
+      ex[u] = tX == f.occ;
+      const bool act = (ex[u] || tX == f.vir) && at + (unsigned int)e < n && !is_dead(st.c[e]);
+      word[u] = 0xFFFFFFFFu;
+      bits[u] = 0u;
+      mu[u] = 0.0;
+      if (act) {
+        const unsigned long long h = KeyOps<KT>::filt_hash(X ^ m);
+        bits[u] = filter_bits(t, h);
+        mu[u] = t.lam[at + (unsigned int)e];
+        if (t.filt) word[u] = t.filt[filter_word(t, h)];
+      }
+    }
+  };
+  unsigned int base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (unsigned int)kRound;
+  stage(0, base);
+  stage(1, base + step);
+  cp_async_wait_all_but_last();
+  __syncwarp();
+  if (base < n) look(0, base);
+  for (int b = 0; base < n; base += step, b = b == 2 ? 0 : b + 1) {
+    const int b1 = b == 2 ? 0 : b + 1, b2 = b1 == 2 ? 0 : b1 + 1;
+    stage(b2, base + 2 * step);
+    cp_async_wait_all_but_last();  // the next round's copy has landed (this lane's pieces)
+    __syncwarp();                  // ... and every other lane's
+    unsigned int wd[kScanTiles], fb[kScanTiles];
+    bool e0[kScanTiles];
+    double mu0[kScanTiles];
+#pragma unroll
+    for (int u = 0; u < kScanTiles; ++u) {
+      wd[u] = word[u];
+      fb[u] = bits[u];
+      e0[u] = ex[u];
+      mu0[u] = mu[u];
+    }
+    if (base + step < n) look(b1, base + step);
+    const ScanStageT<KT>& st = w.stage[b];
+#pragma unroll
+    for (int u = 0; u < kScanTiles; ++u) {
+      const int x = 32 * u + (int)lane;
+      const unsigned int i = base + (unsigned int)x;
+      const bool act = fb[u] != 0u, absent = (wd[u] & fb[u]) != fb[u];
+      const unsigned int ma = __ballot_sync(0xFFFFFFFFu, act), ml = __ballot_sync(0xFFFFFFFFu, act && absent);
+      if (act && absent) {
+        const double x0 = __dmul_rn(st.c[x], f.ic);
+        lone = fma(mu0[u], x0, lone);
+        t.amps[i] = x0;
+        t.lam[i] = __dmul_rn(f.c, mu0[u]);
+      }
+      pairs += __popc(ml);
+      const unsigned int mp = ma & ~ml;
+      if (mp) {
+        enqueue(w.probe, np, mp, below_me, act && !absent, i, st.X[x], st.c[x], e0[u]);
+        np += __popc(mp);
+      }
+    }
+#pragma unroll 1
+    while (np >= 32) drain32(w.probe, np, lane, probe);
+    __syncwarp();  // every lane is done with this buffer before it is refilled
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");  // nothing left in flight
+  if (np > 0) drain_rest(w.probe, np, lane, probe);
 }
 
 // (ab|cd) in chemist notation over spatial orbitals.

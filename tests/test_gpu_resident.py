@@ -177,3 +177,38 @@ def test_batch_mixes_cluster_sizes_and_paths(torch_cuda):
         ref.set_options(rebuild_test_regions=1)
         Er, gr = ref.gradient(eps=1e-7)
         assert abs(e - Er) <= E_TOL and np.max(np.abs(g - gr)) <= G_TOL, n
+
+
+@pytest.mark.parametrize("eps,sigma,angles", [
+    (2.0 ** -12, 0.3, None), (2.0 ** -7, 0.5, None), (1e-6, 0.05, None), (0.02, 1.5, None),
+    (5e-324, 0.1, None), (1e-300, 0.1, None),
+    (2.0 ** -10, 0.1, "exact"), (1e-4, 0.1, "zeros")])
+def test_launch_per_factor_settles_lone_entries_exactly(torch_cuda, eps, sigma, angles):
+    # A launch per factor settles lone entries by the exponents of their
+    # amplitude and sin(theta): thresholds that are powers of two, products that
+    # fall on them, zero angles, large angles, thresholds below every normal
+    # number; counts and amplitudes bit for bit, and the gradient.
+    import oracle
+    from paper_2301_05726_gb300.api import UCCContext
+    p = synth.make_problem(5, 8, 3, 3, sigma, eps=eps).prefix(260)
+    th = p.theta.copy()
+    if angles == "exact":
+        th[::3] = np.arcsin(2.0 ** -5)  # products 2^-5 2^-5 on the threshold 2^-10
+    elif angles == "zeros":
+        th[1::2] = 0.0
+    p = p.with_theta(th)
+    p.eps = eps
+    ok, oa, oc = oracle.Oracle(p).apply()
+    E_o, g_o = oracle.Oracle(p).gradient()
+    ctx = UCCContext(p)
+    ctx.set_options(rebuild_test_regions=1)
+    ctx.apply()
+    st = ctx.stats()
+    same_state(ctx.wavefunction(), (ok, oa))
+    for c in ("rotations", "created", "dropped_new", "dropped_old"):
+        assert st[c] == oc[c], c
+    E, g = ctx.gradient()
+    assert abs(E - E_o) <= E_TOL and np.max(np.abs(g - g_o)) <= G_TOL
+    res = UCCContext(p)  # the resident path takes the same decisions
+    res.apply()
+    same_state(res.wavefunction(), (ok, oa))
