@@ -100,6 +100,26 @@ def test_state_and_gradient(torch_cuda, name):
     assert abs(E - Eg) <= E_TOL and np.max(np.abs(g - gg)) <= G_TOL
 
 
+@pytest.mark.parametrize("name", ["cut_odd", "wide_eps_cut", "grid_cut", "grid_ties"])
+def test_cut_threshold_that_moves(torch_cuda, name):
+    """Angles whose size changes by powers of ten on the way: a cut's threshold
+    lies near the last one's, below its window, above it, or in a bin of ties."""
+    import oracle
+    from paper_2301_05726_gb300.api import UCCContext
+    p = problem(name)
+    scale = np.array([1.0, 1e-3, 1.0, 10.0, 1e-6])[np.arange(p.n_exc) * 5 // p.n_exc]
+    p2 = p.with_theta(np.clip(p.theta * scale, -0.7, 0.7))
+    p2.n_max, p2.n_cut = p.n_max, p.n_cut
+    ok, oa, oc = oracle.Oracle(p2).apply()
+    ctx = UCCContext(p2)
+    ctx.apply()
+    st = ctx.stats()
+    same_state(ctx.wavefunction(), (ok, oa))
+    for c in ("rotations", "created", "dropped_new", "dropped_old", "cut"):
+        assert st[c] == oc[c], c
+    assert st["forward_launches"] == 1 and oc["cut"] > 0
+
+
 @pytest.mark.parametrize("name", ["one_cta_open_shell_eps", "sixteen_ctas", "cut_odd", "grid_cut"])
 def test_entropy(torch_cuda, name):
     import oracle
