@@ -195,11 +195,12 @@ struct ResJob {
 
 // Control words of a resident launch over the whole grid, cleared before it:
 // the barrier's ring, messages received [buffer][kind][CTA] (a sector each),
-// and the cut's histogram and candidates.
+// and the cut's histogram, window counts and candidates.
 struct ResControl {
   unsigned long long words[4][16];
   unsigned int count[2][2][240][8];
   unsigned int hist[4096];
+  unsigned int win[2][516];  // the window's bins and the count above it, two buffers
   unsigned int ncand, pad[3];
   unsigned long long cand_mag[512], cand_key[1024];
 };
