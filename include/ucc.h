@@ -211,8 +211,9 @@ ucc_status ucc_energy(ucc_ctx* ctx, double* E, double* norm2);
  * usable state (a later ucc_energy returns UCC_ESTATE).  Synchronises. */
 ucc_status ucc_gradient(ucc_ctx* ctx, double eps, double* E, double* grad, int on_device);
 
-/* Copy the live determinants of the held state (unordered) into caller
- * buffers of capacity cap: keys (one uint64 per determinant up to 64
+/* Copy the live determinants of the held state into caller buffers
+ * (unordered; host buffers in ascending key order when the device memory for
+ * sorting, twice the keys, can be had) of capacity cap: keys (one uint64 per determinant up to 64
  * spin-orbitals, two -- low word first -- above, so 2*cap words), amps, and
  * optionally sigma = P_S H psi from the last energy evaluation (NULL to
  * skip).  Host or device pointers (on_device).  *n receives the count;

@@ -133,9 +133,13 @@ class UCCContext:
                                             sig.ctypes.data_as(ctypes.c_void_p) if with_sigma else None, 0))
         if self.key_words == 2:
             keys = keys.reshape(cap, 2)
-            order = np.lexsort((keys[:, 0], keys[:, 1]))
+            lo, hi = keys[:, 0], keys[:, 1]
+            ascending = np.all((hi[1:] > hi[:-1]) | ((hi[1:] == hi[:-1]) & (lo[1:] > lo[:-1])))
+            order = None if ascending else np.lexsort((lo, hi))
         else:
-            order = np.argsort(keys, kind="stable")
+            order = None if np.all(keys[1:] > keys[:-1]) else np.argsort(keys, kind="stable")
+        if order is None:  # the library sorts where it has the memory for it
+            return (keys, amps, sig) if with_sigma else (keys, amps)
         if with_sigma:
             return keys[order], amps[order], sig[order]
         return keys[order], amps[order]

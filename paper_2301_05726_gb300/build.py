@@ -19,7 +19,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libucc.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["ucc_api.cu", "k_apply.cu", "k_energy.cu", "k_sigma_bucket.cu", "k_adjoint.cu", "k_select.cu", "k_batch.cu", "k_persist.cu",
-           "k_resident.cu", "ucc_static.cu"]
+           "k_resident.cu", "k_sort.cu", "ucc_static.cu"]
 HEADERS = ["ucc_internal.h", "ucc_device.cuh", "ucc_steps.cuh", "ucc_keys.cuh"]
 
 

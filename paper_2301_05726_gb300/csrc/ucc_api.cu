@@ -2169,6 +2169,38 @@ ucc_status batch_together(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
   return s;
 }
 
+// The held state to host buffers in key order.  UCC_ENOMEM: no memory to sort in.
+template <class KT>
+ucc_status export_sorted(ucc_ctx* c, TableSet& tab, unsigned long long live, uint64_t* keys, double* amps,
+                         double* sigma) {
+  if (live >> 32) return UCC_ENOMEM;  // (positions are 32-bit)
+  unsigned char* buf = nullptr;
+  const size_t words = sort_scratch_words(live);
+  UCC_TRY(dalloc(&buf, live * (2 * sizeof(KT) + 2 * sizeof(double) + 2 * sizeof(unsigned int)) +
+                           words * sizeof(unsigned int)));
+  SortListT<KT> a, b;
+  a.keys = reinterpret_cast<KT*>(buf);
+  b.keys = a.keys + live;
+  double* const da = reinterpret_cast<double*>(b.keys + live);
+  double* const ds = da + live;
+  a.idx = reinterpret_cast<unsigned int*>(ds + live);
+  b.idx = a.idx + live;
+  const KT* sorted = nullptr;
+  const ucc_status s = [&]() -> ucc_status {
+    CUDA_TRY(cudaMemsetAsync(&tab.d_cnt->new_n, 0, sizeof(unsigned long long), c->stream));
+    CUDA_TRY(launch_sorted_export(c->template table<KT>(tab), live, c->n_so, a, b, b.idx + live, da,
+                                  sigma ? ds : nullptr, c->full_grid(), c->stream, &sorted));
+    CUDA_TRY(cudaMemcpyAsync(keys, sorted, live * sizeof(KT), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(amps, da, live * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    if (sigma) CUDA_TRY(cudaMemcpyAsync(sigma, ds, live * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    return read_counters(c, tab);
+  }();
+  dfree(buf);
+  UCC_TRY(s);
+  if (tab.h_cnt->new_n != live) return fail(UCC_ECUDA, "export count mismatch");
+  return UCC_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -2340,6 +2372,9 @@ ucc_status ucc_get_wavefunction(ucc_ctx* c, size_t cap, size_t* n, uint64_t* key
   double* ta = nullptr;
   double* tsig = nullptr;
   if (!on_device) {
+    const ucc_status s = c->wide ? export_sorted<Key128>(c, tab, live, keys, amps, sigma)
+                                 : export_sorted<unsigned long long>(c, tab, live, keys, amps, sigma);
+    if (s != UCC_ENOMEM) return s;
     UCC_TRY(dalloc(&tk, live * c->kw));
     UCC_TRY(dalloc(&ta, live));
     if (sigma) UCC_TRY(dalloc(&tsig, live));

@@ -357,6 +357,19 @@ cudaError_t launch_finish_rebuild(const TableT<KT>& t, unsigned long long expect
 template <class KT>
 cudaError_t launch_export(const TableT<KT>& t, unsigned long long cap, KT* keys, double* amps, double* sigma,
                           int grid, cudaStream_t st);
+// The n live entries in ascending key order: amps and sigma (may be null) are
+// written, *sorted is the keys' list (one of a and b, n entries each).  scratch:
+// sort_scratch_words(n) words; t.cnt->new_n is zero and counts the live entries.
+template <class KT>
+struct SortListT {
+  KT* keys;
+  unsigned int* idx;
+};
+size_t sort_scratch_words(unsigned long long n);
+template <class KT>
+cudaError_t launch_sorted_export(const TableT<KT>& t, unsigned long long n, int key_bits, SortListT<KT> a,
+                                 SortListT<KT> b, unsigned int* scratch, double* amps, double* sigma, int grid,
+                                 cudaStream_t st, const KT** sorted);
 template <class KT>
 cudaError_t launch_sigma(const TableT<KT>& t, const Integrals& in, int grid, cudaStream_t st);
 template <class KT>
