@@ -212,20 +212,18 @@ __global__ void __launch_bounds__(kThreads) k_rehash(TableT<KT> t) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       h[u] = home_slot(t, key[u]);
-      prev[u] = !K::is_zero(key[u]) ? key_cas(&t.slots[h[u]].key, K::zero(), key[u]) : K::bit(0);
+      prev[u] = !K::is_zero(key[u]) ? slot_cas(&t.slots[h[u]], key[u], i0 + u * stride) : K::bit(0);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (K::is_zero(key[u])) continue;
-      const unsigned long long i = i0 + u * stride;
-      unsigned long long s = h[u];
       if (K::is_zero(prev[u])) {
         filter_add(t, key[u]);
       } else {
         if (prev[u] == key[u]) raise_consistency(t.cnt, SITE_REHASH_DUP, K::lo(key[u]));
-        s = claim_slot(t, key[u], h[u] + 1);
+        const unsigned long long s = claim_slot(t, key[u], h[u] + 1);
+        if (s != ~0ull) t.slots[s].idx = i0 + u * stride;
       }
-      if (s != ~0ull) t.slots[s].idx = i;
     }
   }
 }

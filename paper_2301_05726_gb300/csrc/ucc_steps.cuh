@@ -137,9 +137,8 @@ template <class KT>
 __device__ __forceinline__ void link_appended(const TableT<KT>& t, KT key, unsigned long long idx) {
   unsigned long long h = home_slot(t, key);
   for (int step = 0; step < MAX_PROBE; ++step) {
-    const KT prev = key_cas(&t.slots[h].key, KeyOps<KT>::zero(), key);
+    const KT prev = slot_cas(&t.slots[h], key, idx);
     if (KeyOps<KT>::is_zero(prev)) {
-      t.slots[h].idx = idx;
       filter_add(t, key);
       return;
     }
@@ -156,9 +155,8 @@ __device__ __forceinline__ void link_from_slot(const TableT<KT>& t, KT key, unsi
                                                unsigned long long start) {
   unsigned long long h = start & t.slot_mask;
   for (int step = 0; step < MAX_PROBE; ++step) {
-    const KT prev = key_cas(&t.slots[h].key, KeyOps<KT>::zero(), key);
+    const KT prev = slot_cas(&t.slots[h], key, idx);
     if (KeyOps<KT>::is_zero(prev)) {
-      t.slots[h].idx = idx;
       filter_add(t, key);
       return;
     }
