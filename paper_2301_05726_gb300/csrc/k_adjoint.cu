@@ -140,8 +140,12 @@ __global__ void __launch_bounds__(kThreads) k_link_tail(TableT<KT> t) {
     link_appended(t, t.keys[j], j);
 }
 
+// Seven blocks per SM: held to the 64 registers of eight, a step takes 4 % longer
+// (the reverse sweep of the 64-spin-orbital problem at N_MAX 1e7: 276 and 264 ms);
+// with six it takes 1 % longer.  FP64 (16 cycles per warp instruction) and random
+// sectors bound it together, each at some 55 % of its rate.
 template <class KT, int G>
-__global__ void __launch_bounds__(kStepThreads, 8) k_reverse(TableT<KT> t, const FactorT<KT>* __restrict__ factors,
+__global__ void __launch_bounds__(kStepThreads, 7) k_reverse(TableT<KT> t, const FactorT<KT>* __restrict__ factors,
                                                              int k, unsigned int stamp, double* grad) {
   __shared__ ReverseScratchT<KT> s_w[kStepThreads / 32];
   const FactorT<KT> f = factors[k];
