@@ -192,7 +192,6 @@ struct ucc_ctx {
   // Bucketed energy: per-partition counts, fill counters and offsets, and the
   // record buffer (kept between evaluations).
   unsigned int* d_sb_cnt = nullptr;
-  unsigned int* d_sb_fill = nullptr;
   unsigned long long* d_sb_off = nullptr;
   unsigned long long sb_parts = 0;
   unsigned char* d_sb_rec = nullptr;
@@ -1158,13 +1157,10 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
   };
   if (c->sb_parts < P) {
     dfree(c->d_sb_cnt);
-    dfree(c->d_sb_fill);
     dfree(c->d_sb_off);
     c->sb_parts = 0;
-    if (dalloc(&c->d_sb_cnt, P) != UCC_OK || dalloc(&c->d_sb_fill, P) != UCC_OK ||
-        dalloc(&c->d_sb_off, sb_offsets(P)) != UCC_OK) {
+    if (dalloc(&c->d_sb_cnt, P) != UCC_OK || dalloc(&c->d_sb_off, sb_offsets(P)) != UCC_OK) {
       dfree(c->d_sb_cnt);
-      dfree(c->d_sb_fill);
       dfree(c->d_sb_off);
       return unavailable("partition arrays");
     }
@@ -1182,7 +1178,7 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
     if (bytes < 32 * rec_bytes || dalloc(&c->d_sb_rec, bytes) != UCC_OK) return unavailable("record buffer");
     c->sb_rec_cap = bytes;
   }
-  unsigned long long cap_recs = c->sb_rec_cap / rec_bytes;
+  unsigned long long cap_recs = std::min<unsigned long long>(c->sb_rec_cap / rec_bytes, 0xFFFFFFFFull);
   if (c->opt.energy_test_buffer_records > 0)
     cap_recs = std::min<unsigned long long>(cap_recs, (unsigned long long)c->opt.energy_test_buffer_records);
   const int grid = (int)std::max<unsigned long long>(
@@ -1225,10 +1221,10 @@ ucc_status energy_by_buckets(ucc_ctx* c, TableSet& s, const Integrals& in, bool*
       continue;
     }
     if (b == a) continue;
-    CUDA_TRY(cudaMemsetAsync(c->d_sb_fill + p0, 0, (p1 - p0) * sizeof(unsigned int), c->stream));
-    CUDA_TRY(launch_sb_scatter(t, c->d_sb_off, c->d_sb_fill, rec, pt, p0, p1, a, grid, c->stream));
+    CUDA_TRY(launch_sb_scatter(t, c->d_sb_off, c->d_sb_cnt, rec, pt, p0, p1, a, (unsigned int)(b - a), grid,
+                               c->stream));
     CUDA_TRY(launch_sb_pairs(t, in, rec, c->d_sb_off, pt, p0, p1, a, pair_grid, c->stream));
-    c->launches += 3;
+    c->launches += 4;
   }
   CUDA_TRY(launch_sb_finish(t, in, grid, c->stream));
   c->launches++;
@@ -1546,7 +1542,6 @@ void destroy(ucc_ctx* c) {
   dfree(c->d_grad);
   dfree(c->d_partials);
   dfree(c->d_sb_cnt);
-  dfree(c->d_sb_fill);
   dfree(c->d_sb_off);
   dfree(c->d_sb_rec);
   dfree(c->d_res_ctl);

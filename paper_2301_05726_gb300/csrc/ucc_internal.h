@@ -375,15 +375,15 @@ cudaError_t launch_sigma(const TableT<KT>& t, const Integrals& in, int grid, cud
 template <class KT>
 cudaError_t launch_lambda_init(const TableT<KT>& t, int grid, cudaStream_t st);
 // Bucketed energy: records per core partition, their prefix sum, the records
-// of partitions [p0, p1) (fill: per-partition counters, zeroed per round),
-// the pair sums into sigma, and the diagonal with E and <psi|psi>.
+// of partitions [p0, p1) (`records` of them; next: where a partition's next one
+// goes, the counts' array used again), the pair sums into sigma, and the diagonal with E and <psi|psi>.
 template <class KT>
 cudaError_t launch_sb_count(const TableT<KT>& t, unsigned int* cnt, SbParts pt, int grid, cudaStream_t st);
 cudaError_t launch_sb_scan(const unsigned int* cnt, unsigned long long* off, unsigned long long n, cudaStream_t st);
 template <class KT>
-cudaError_t launch_sb_scatter(const TableT<KT>& t, const unsigned long long* off, unsigned int* fill,
+cudaError_t launch_sb_scatter(const TableT<KT>& t, const unsigned long long* off, unsigned int* next,
                               SigRecT<KT>* rec, SbParts pt, unsigned long long p0, unsigned long long p1,
-                              unsigned long long base, int grid, cudaStream_t st);
+                              unsigned long long base, unsigned int records, int grid, cudaStream_t st);
 template <class KT>
 cudaError_t launch_sb_pairs(const TableT<KT>& t, const Integrals& in, const SigRecT<KT>* rec,
                             const unsigned long long* off, SbParts pt, unsigned long long p0, unsigned long long p1,
