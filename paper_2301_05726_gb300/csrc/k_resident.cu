@@ -90,7 +90,7 @@ __host__ __device__ inline unsigned int up16(unsigned int x) { return (x + 15u) 
 
 // Byte offsets of a CTA's shared arrays, host and device.
 struct ResLayout {
-  unsigned int keys, amps, lam, born, slots, queue, done, hist, comb, cmag, ckey, win, stage, inkey, ina, inb, bytes;
+  unsigned int keys, amps, lam, born, slots, queue, done, hist, comb, cmag, ckey, win, ent, stage, inkey, ina, inb, bytes;
 };
 
 template <class KT>
@@ -121,6 +121,7 @@ __host__ __device__ inline ResLayout res_layout(const ResGeom& g, bool reverse) 
     o.win = take(g.grid ? 0u : (unsigned int)g.ctas * kWinBins * 2u);
     o.cmag = take(kCand * 8u);
     o.ckey = take((unsigned int)(kCand * sizeof(KT)));
+    o.ent = take(g.entropy ? L * 8u : 0u);
   }
   o.bytes = at;
   return o;
@@ -306,6 +307,7 @@ struct ResView {
   KT* keys;
   double* amps;
   double* lam;
+  double* ent;  // the entries' terms of the entropy (null: not recorded)
   unsigned int* born;
   unsigned int* slots;
   unsigned short* queue;
@@ -322,6 +324,7 @@ __device__ __forceinline__ ResView<KT> res_view(unsigned char* smem, const ResLa
   v.keys = reinterpret_cast<KT*>(smem + o.keys);
   v.amps = reinterpret_cast<double*>(smem + o.amps);
   v.lam = reverse ? reinterpret_cast<double*>(smem + o.lam) : nullptr;
+  v.ent = !reverse && g.entropy ? reinterpret_cast<double*>(smem + o.ent) : nullptr;
   v.born = reinterpret_cast<unsigned int*>(smem + o.born);
   v.slots = reinterpret_cast<unsigned int*>(smem + o.slots);
   v.queue = reinterpret_cast<unsigned short*>(smem + o.queue);
@@ -433,7 +436,7 @@ __device__ __forceinline__ void res_insert(const ResView<KT>& v, KT key, unsigne
 // entry is still being written.
 template <class KT>
 __device__ __forceinline__ bool res_append(const ResView<KT>& v, KT key, double a, unsigned int born,
-                                           unsigned int* tail) {
+                                           unsigned int* tail, double ent = 0.0) {
   cg::coalesced_group g = cg::coalesced_threads();
   unsigned int i = 0u;
   if (g.thread_rank() == 0) i = atomicAdd(tail, (unsigned int)g.size());
@@ -443,6 +446,7 @@ __device__ __forceinline__ bool res_append(const ResView<KT>& v, KT key, double 
   v.amps[i] = a;
   v.born[i] = born;
   if (v.lam) v.lam[i] = 0.0;
+  if (v.ent) v.ent[i] = ent;
   return true;
 }
 
@@ -477,6 +481,7 @@ __device__ __forceinline__ unsigned int res_compact(const ResView<KT>& v, unsign
       key = v.keys[i];
       born = v.born[i];
       if (v.lam) lam = v.lam[i];
+      if (v.ent) lam = v.ent[i];  // (never both)
     }
     const bool kp = live && keep(a, key);
     const unsigned int mk = __ballot_sync(0xFFFFFFFFu, kp), md = __ballot_sync(0xFFFFFFFFu, live && !kp);
@@ -498,6 +503,7 @@ __device__ __forceinline__ unsigned int res_compact(const ResView<KT>& v, unsign
       v.amps[to] = a;
       v.born[to] = born;
       if (v.lam) v.lam[to] = lam;
+      if (v.ent) v.ent[to] = lam;
     } else if (live) {
       drop(key, a, born, dropped + pd + __popc(md & below_me));
     }
@@ -576,6 +582,7 @@ __device__ __forceinline__ bool res_load(const ResView<KT>& v, Net& net, const T
     v.amps[j] = t.amps[i];
     v.born[j] = t.born[i];
     if (v.lam) v.lam[j] = t.lam[i];
+    if (v.ent) v.ent[j] = entropy_term(v.amps[j]);
   };
   bool ok = true;
   if constexpr (Net::kGrid) {
@@ -1098,7 +1105,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
   Window win{false, 0ull, 0};
   Counters* const cnt = job.t.cnt;
   const unsigned int tid = threadIdx.x, lane = tid & 31u;
-  const bool ent = job.t.entropy != nullptr;
+  const bool ent = v.ent != nullptr && job.t.entropy != nullptr;
   double dS_due = 0.0;  // this thread's share of the last factor's change of the entropy
 
   if (tid == 0) {
@@ -1151,6 +1158,15 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
       raise_error(cnt, ERR_TAPE_FULL);
     }
     atomicAdd(&s_drop, 1u);
+  };
+
+  // What entry at's new amplitude changes in the entropy; its old term is kept, so
+  // a rotation takes one logarithm (with the old term taken anew, the 315 factors of
+  // 3,136 determinants at 16 spin-orbitals: 2.2 ms, so 1.8).
+  auto new_term = [&](int at, double c, bool out) {
+    const double was = v.ent[at], now = out ? 0.0 : entropy_term(c);
+    v.ent[at] = now;
+    return now - was;
   };
 
   while (k < job.k1) {
@@ -1208,7 +1224,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
         atomicOr(&v.done[at >> 5], 1u << (at & 31));
         rot += zE;
         const bool out = below_eps(nZ, job.eps);
-        if (ent) dS += (out ? 0.0 : entropy_term(nZ)) - entropy_term(cZ);
+        if (ent) dS += new_term(at, nZ, out);
         if (out) {
           if (RECORD) record(Z, nZ, v.born[at]);
           v.amps[at] = dead_value(stamp);
@@ -1224,13 +1240,15 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
           ++dnew;
           continue;
         }
-        if (ent) dS += entropy_term(nZ);
+        double eZ = 0.0;
+        if (ent) dS += eZ = entropy_term(nZ);
         ++cre;
         if (at >= 0) {  // a dropped entry comes back
+          if (ent) v.ent[at] = eZ;
           v.amps[at] = nZ;
           v.born[at] = (unsigned int)k;
           atomicSub(&s_dead, 1u);
-        } else if (!res_append(v, Z, nZ, (unsigned int)k, &s_tail)) {
+        } else if (!res_append(v, Z, nZ, (unsigned int)k, &s_tail, eZ)) {
           s_full = 1;
         }
       }
@@ -1250,7 +1268,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
       }
       ++rot;
       const bool out = below_eps(nX, job.eps);
-      if (ent) dS += (out ? 0.0 : entropy_term(nX)) - entropy_term(cX);
+      if (ent) dS += new_term((int)i, nX, out);
       if (out) {
         if (RECORD) record(v.keys[i], nX, v.born[i]);
         v.amps[i] = dead_value(stamp);
@@ -1654,13 +1672,14 @@ cudaError_t res_launch(Kernel kernel, const ResJob<KT>& one, const ResJob<KT>* m
 // (inside a cluster the inboxes lie there too).
 constexpr int kMostCluster[3] = {0, 2048, 1792}, kMostGrid[3] = {0, 5632, 4352};
 
-ResGeom shape(int ctas, bool grid, double L, int key_words) {
+ResGeom shape(int ctas, bool grid, double L, bool entropy, int key_words) {
   ResGeom g{};
   g.ctas = ctas;
   g.grid = grid ? 1 : 0;
   const int most = grid ? kMostGrid[key_words] : kMostCluster[key_words];
   g.L = std::max(256, std::min(most, ((int)L + 31) / 32 * 32));
   g.Lin = g.L;
+  g.entropy = entropy ? 1 : 0;
   g.logB = 4;  // buckets of four slots, at most three quarters full
   while (3 * (4 << g.logB) < 4 * g.L) ++g.logB;
   return g;
@@ -1673,7 +1692,7 @@ ResLimits find_limits() {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   for (int ctas = kMaxC; ctas >= 1 && r.cluster == 0; ctas /= 2) {
-    const ResGeom g = shape(ctas, false, kMostCluster[kw], kw);
+    const ResGeom g = shape(ctas, false, kMostCluster[kw], true, kw);
     int n[2] = {0, 0};
     if (res_config(k_res_forward<KT, true, ClusterNet<KT>>, KT{}, 1, g, false, nullptr, &cfg, attr) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&n[0], k_res_forward<KT, true, ClusterNet<KT>>, &cfg) == cudaSuccess &&
@@ -1684,7 +1703,7 @@ ResLimits find_limits() {
     cudaGetLastError();
   }
   int dev = 0, sms = 0, coop = 0, a = 0, b = 0;
-  const ResGeom g = shape(1, true, kMostGrid[kw], kw);
+  const ResGeom g = shape(1, true, kMostGrid[kw], true, kw);
   if (cudaGetDevice(&dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
@@ -1711,24 +1730,29 @@ bool res_room(unsigned long long entries, const ResGeom& g) {
   return entries < (1ull << 20) && largest_share((float)entries, g.ctas) <= (float)g.L;
 }
 
-bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, ResGeom* g) {
+bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, bool entropy, ResGeom* g) {
   if (max_ctas < 1) return false;
-  int ctas = most <= 512 ? 1 : most <= 2048 ? 4 : most <= 6144 ? 8 : 16;
+  // A recorded entropy takes a logarithm per rotation, some eighty FP64
+  // instructions of 16 cycles a warp: its SMs are worth more than its barriers cost
+  // (a factor at 100, 1,225 and 3,136 determinants: 5.5, 4.9 and 4.9 us with the
+  // clusters of the other runs, 4.8, 4.7 and 4.7 with sixteen; the whole GPU: 6.0,
+  // 5.7, 5.8).
+  int ctas = entropy ? kMaxC : most <= 512 ? 1 : most <= 2048 ? 4 : most <= 6144 ? 8 : 16;
   ctas = std::min(ctas, max_ctas);
   for (; ctas <= max_ctas; ctas *= 2) {
     // a quarter more than the largest share, for dropped entries and inboxes
     const double want = 1.25 * (double)largest_share((float)most, ctas) + 32.0;
     if (want <= (double)kMostCluster[key_words]) {
-      *g = shape(ctas, false, want, key_words);
+      *g = shape(ctas, false, want, entropy, key_words);
       return true;
     }
   }
   return false;
 }
 
-bool res_grid_shape(unsigned long long most, int key_words, int ctas, ResGeom* g) {
+bool res_grid_shape(unsigned long long most, int key_words, int ctas, bool entropy, ResGeom* g) {
   if (ctas < 1) return false;
-  *g = shape(ctas, true, 1.25 * (double)largest_share((float)most, ctas) + 32.0, key_words);
+  *g = shape(ctas, true, 1.25 * (double)largest_share((float)most, ctas) + 32.0, entropy, key_words);
   return true;
 }
 

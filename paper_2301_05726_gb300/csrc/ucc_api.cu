@@ -614,7 +614,9 @@ bool resident_shape(const ucc_ctx* c, ResGeom* g) {
   if (c->opt.rebuild_test_regions != 0 || c->opt.probe_width != 0 || c->opt.max_entries > 0) return false;
   const ResLimits lim = res_limits(c->kw);
   const unsigned long long most = most_entries(c);
-  return res_cluster_shape(most, c->kw, lim.cluster, g) || res_grid_shape(most, c->kw, lim.grid, g);
+  const bool entropy = c->opt.record_entropy != 0;
+  return res_cluster_shape(most, c->kw, lim.cluster, entropy, g) ||
+         res_grid_shape(most, c->kw, lim.grid, entropy, g);
 }
 
 // Entries a table needs in global memory for what a resident pass can write back.
@@ -1660,7 +1662,8 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
   // sixteen, which pays from ten jobs on (nine large clusters fill the GPU).
   const int lim = res_limits(1).cluster;
   ResGeom g{};
-  if (!(n > 9 && res_cluster_shape(most, 1, std::min(lim, 8), &g)) && !res_cluster_shape(most, 1, lim, &g))
+  if (!(n > 9 && res_cluster_shape(most, 1, std::min(lim, 8), false, &g)) &&
+      !res_cluster_shape(most, 1, lim, false, &g))
     return fail(UCC_ECUDA, "no cluster shape for a batch that has one");
   ResJob<KT>* d_jobs = nullptr;
   JobView* d_view = nullptr;

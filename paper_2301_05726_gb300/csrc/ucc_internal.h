@@ -178,6 +178,7 @@ static_assert(sizeof(SigRecT<unsigned long long>) == 32, "record is one sector")
 // messages and 2^logB hash buckets of four slots.
 struct ResGeom {
   int ctas, grid, L, Lin, logB;
+  int entropy;  // room for the entries' terms of the entropy too
 };
 
 // One job of a resident launch: factors [k0, k1) of a table that holds at most
@@ -434,8 +435,8 @@ int persist_grid(int record, int probe_width, int reverse);
 // (false: too large); res_grid_shape: the whole grid, sized for them as far as
 // it goes; res_room: whether a shape holds that many.
 ResLimits res_limits(int key_words);
-bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, ResGeom* g);
-bool res_grid_shape(unsigned long long most, int key_words, int ctas, ResGeom* g);
+bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, bool entropy, ResGeom* g);
+bool res_grid_shape(unsigned long long most, int key_words, int ctas, bool entropy, ResGeom* g);
 bool res_room(unsigned long long entries, const ResGeom& g);
 // many: n_jobs jobs in device memory, or null for the single job `one`.
 template <class KT>

@@ -132,6 +132,21 @@ def test_entropy(torch_cuda, name):
     assert np.max(np.abs(ctx.entropy() - S)) <= 1e-10
 
 
+@pytest.mark.parametrize("name", ["one_cta", "drops_and_revivals", "wide_eps_cut", "grid_drops_and_revivals"])
+def test_entropy_of_revived_entries(torch_cuda, name):
+    """The kept terms of entries that are dropped, come back, move in a
+    compaction or are cut."""
+    import oracle
+    from paper_2301_05726_gb300.api import UCCContext
+    p = problem(name)
+    ctx = UCCContext(p)
+    ctx.set_options(record_entropy=1)
+    ctx.apply()
+    assert ctx.stats()["forward_launches"] == 1
+    S = oracle.Oracle(p).entropy_per_factor(n_max=p.n_max, n_cut=p.n_cut)
+    assert np.max(np.abs(ctx.entropy() - S)) <= 1e-10
+
+
 def test_outgrows_the_gpu(torch_cuda):
     # Resident to begin with; past some 700,000 determinants a launch per factor.
     from paper_2301_05726_gb300.api import UCCContext
