@@ -255,7 +255,7 @@ def flush_l2(buf):
 # entries per launch, far larger than L2; the summary under profiles/ gives the command); a full-size
 # launch's traffic is taken as this figure times the entries it scans.  A kernel is left out (traffic
 # reported as null) once its code has changed since its capture.
-TRAFFIC_PER_SCANNED_ENTRY = {"k_reverse": 47.3}
+TRAFFIC_PER_SCANNED_ENTRY = {"k_reverse": 45.5}
 
 
 def _roofline(kernel, bytes_, ms, launches, hbm, peak_kind, scanned=0):
@@ -386,7 +386,7 @@ def n1_leg(args):
 def batch_leg(args):
     """The 256-job workload (16-36 spin-orbitals, 4-12 electrons, theta ~ N(0, 0.02), eps = 1e-8), each
     job with the paper's production cut (N_MAX = 8,000, N_CUT = 5,000): energies and adjoint gradients
-    of all jobs through one ucc_batch_run call (persistent launches), and the same for a sample of jobs
+    of all jobs through one ucc_batch_run call, and the same for a sample of jobs
     against the one-job path."""
     import torch
     from paper_2301_05726_gb300 import synth

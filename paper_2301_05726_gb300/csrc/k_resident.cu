@@ -22,10 +22,10 @@
 // by the same formulas; the only traffic is one message per linked entry and
 // the only wait one barrier (inboxes alternate between two buffers).  When the
 // step might leave more than N_MAX determinants (the barrier's sums say so) a
-// second barrier counts them, and a cut follows: a histogram of |c| (4,096 bins
-// over the exponents that amplitudes have) summed over the CTAs, and a pairwise
-// rank of the few entries of the threshold's bin.  Dropping, compacting and
-// rehashing are each CTA's own business.  The reverse sweep has the same two
+// second barrier counts them, with the entries binned around the last cut's
+// threshold, and a cut follows: the few entries of the threshold's bin are ranked
+// pairwise (a first cut takes a histogram of |c|, 4,096 bins over the exponents that
+// amplitudes have).  Dropping, compacting and rehashing are each CTA's own business.  The reverse sweep has the same two
 // phases; factor k - 1's tape records travel with factor k's messages.
 //
 // Inside a cluster messages are remote shared-memory stores and the barrier is
@@ -37,12 +37,12 @@
 // across the GPU), of a message (0.5 and 1 us) and of the block's own phases.
 // Times before (a launch per factor) and with it: a factor of the 64-spin-
 // orbital, 10-electron problem at N_MAX 8,000 (6,000 keys scanned, 2,400 pairs, a
-// cut after every other factor) 74 and 8.8 us forward, 51 and 7.9 us reverse, the
-// gradient's 5,270 factors 659 and 89 ms (72 spin-orbitals, two-word keys: 726 and
-// 100); N_MAX 160,000, a factor and its cuts 78 and 14 us; 245,025 determinants
-// at 24 spin-orbitals, a factor 23.6 and 5.5 us forward, 18 and 7.1 reverse;
-// 621,075 at 30, 23.8 and 7.0 us; 24 uneven jobs in one batch, a cluster each,
-// 646 and 37 ms; 12 spin-orbitals (225 determinants, one CTA), 2.44 and 0.93 ms.
+// cut after every other factor) 74 and 7.6 us forward, 51 and 7.9 us reverse, the
+// gradient's 5,270 factors 655 and 82 ms (72 spin-orbitals, two-word keys: 709 and
+// 93); N_MAX 160,000, a factor and its cuts 78 and 11.7 us; 245,025 determinants
+// at 24 spin-orbitals, a factor 23.6 and 5.8 us forward, 18 and 7.2 reverse;
+// 621,075 at 30, 23.8 and 7.4 us; 24 uneven jobs in one batch, a cluster each,
+// 664 and 36 ms; 12 spin-orbitals (225 determinants, one CTA), 2.50 and 0.85 ms.
 //
 // The arithmetic, the eps rule, the cut's order and the counts are those of the
 // launch-per-factor kernels, so states agree bit for bit.
