@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(kThreads) k_rehash(TableT<KT> t) {
         filter_add(t, key[u]);
       } else {
         if (prev[u] == key[u]) raise_consistency(t.cnt, SITE_REHASH_DUP, K::lo(key[u]));
-        const unsigned long long s = claim_slot(t, key[u], h[u] + 1);
-        if (s != ~0ull) t.slots[s].idx = i0 + u * stride;
+        // (not claim_slot: every claim of a launch has one size)
+        claim_slot_for(t, key[u], i0 + u * stride, h[u] + 1, SITE_DUP_CLAIM);
       }
     }
   }

@@ -284,6 +284,26 @@ __device__ __forceinline__ unsigned long long claim_slot(const TableT<KT>& t, KT
   return ~0ull;
 }
 
+// The same for a key whose entry is known: key and index enter the slot together.
+template <class KT>
+__device__ __forceinline__ void claim_slot_for(const TableT<KT>& t, KT key, unsigned long long idx,
+                                               unsigned long long start, int site) {
+  unsigned long long h = start & t.slot_mask;
+  for (int step = 0; step < MAX_PROBE; ++step) {
+    const KT prev = slot_cas(&t.slots[h], key, idx);
+    if (KeyOps<KT>::is_zero(prev)) {
+      filter_add(t, key);
+      return;
+    }
+    if (prev == key) {
+      raise_consistency(t.cnt, site, KeyOps<KT>::lo(key));
+      return;
+    }
+    h = (h + 1) & t.slot_mask;
+  }
+  raise_error(t.cnt, ERR_PROBE_BOUND);
+}
+
 // Warp-aggregated increment of a device counter: the lanes that reach this
 // call together share one atomicAdd and receive consecutive values.
 __device__ __forceinline__ unsigned long long aggregated_add(unsigned long long* counter) {
