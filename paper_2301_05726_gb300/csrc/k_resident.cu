@@ -1521,12 +1521,17 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
     if (tid == 0) s_qn = 0u;  // (every thread has its length)
     Msg<KT> msg = net.template get<true>(buf, 0, min(tid, net.Lin - 1u));
     Msg<KT> rec = net.template get<true>(buf, 1, min(tid, net.Lin - 1u));
-    const unsigned int got = net.received(buf, 0), recs = net.received(buf, 1);
-    if (got + recs > net.Lin) s_full = 1;
+    unsigned int got = net.received(buf, 0), recs = net.received(buf, 1);
+    if (got + recs > net.Lin) {
+      // The two kinds have overwritten each other: none is read (what a place holds
+      // may be of either kind), and the next barrier ends the launch.
+      s_full = 1;
+      got = recs = 0u;
+    }
     acc = 0.0;
     if (sweep) {
       const unsigned int stamp = 0x80000000u | (unsigned int)k;
-      for (unsigned int x = tid; x < min(got, net.Lin); x += kT) {
+      for (unsigned int x = tid; x < got; x += kT) {
         if (x != tid) msg = net.template get<true>(buf, 0, x);
         const KT Z = msg.key;
         const int at = res_find(v, Z);
@@ -1570,7 +1575,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
       }
     }
     // The records of factor k - 1: a key that is still stored was dropped.
-    for (unsigned int x = tid; x < min(recs, net.Lin); x += kT) {
+    for (unsigned int x = tid; x < recs; x += kT) {
       if (x != tid) rec = net.template get<true>(buf, 1, x);
       const int at = res_find(v, rec.key);
       if (at >= 0) {

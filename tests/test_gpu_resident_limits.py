@@ -1,0 +1,60 @@
+"""Where a resident pass meets a limit -- an inbox, its room, the tape, memory, a
+wait -- the call gives what a launch per factor gives: energies within 1e-10 Ha,
+gradients within 1e-8, and the same determinants, amplitudes and counts.
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2301_05726_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+E_TOL = 1e-10
+G_TOL = 1e-8
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_05726_gb300 import build
+    build.build()
+    return torch
+
+
+def doubling(n_factors, extra=()):
+    """Singles of distinct electrons into distinct orbitals of 20, so that every factor doubles the
+    table (2^20 determinants after all of them), then the rows of extra."""
+    n, half = 20, 10
+    rng = np.random.default_rng(5)
+    h, g = synth.make_integrals(rng, n)
+    rows = [(2 * i + s, -1, 2 * (i + half) + s, -1) for s in (0, 1) for i in range(half)][:n_factors]
+    exc = np.array(rows + list(extra), dtype=np.int32)
+    return synth.Problem(n, half, half, h, g, exc, rng.uniform(0.15, 0.35, len(exc)), eps=0.0)
+
+
+def context(p, **options):
+    from paper_2301_05726_gb300.api import UCCContext
+    c = UCCContext(p)
+    c.set_options(**options)
+    return c
+
+
+def assert_gradient(got, p, **options):
+    E, g = got
+    Er, gr = context(p, rebuild_test_regions=1, **options).gradient()  # a launch per factor
+    assert abs(E - Er) <= E_TOL and np.max(np.abs(g - gr)) <= G_TOL
+
+
+@pytest.mark.parametrize("n_cut", [100_000, 350_000])
+def test_reverse_meets_a_cut_larger_than_the_inboxes(torch_cuda, n_cut):
+    # The cut after the last single drops more determinants than the GPU's inboxes
+    # take together (or than they take beside the messages of the factor after it),
+    # while the final state is small.
+    p = doubling(20, extra=[(0, 1, 20, 21), (2, 3, 22, 23)])
+    p = dataclasses.replace(p, n_max=1_000_000, n_cut=n_cut)
+    ctx = context(p)
+    assert_gradient(ctx.gradient(), p)
+    assert ctx.stats()["cut"] >= (1 << 20) - n_cut
