@@ -1630,12 +1630,41 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
   net.leave();
 }
 
+// Entries a CTA holds at most: what fits its shared memory in either kernel
+// (inside a cluster the inboxes lie there too).
+constexpr int kMostCluster[3] = {0, 2048, 1792}, kMostGrid[3] = {0, 5632, 4352};
+
+ResGeom shape(int ctas, bool grid, double L, bool entropy, int key_words) {
+  ResGeom g{};
+  g.ctas = ctas;
+  g.grid = grid ? 1 : 0;
+  const int most = grid ? kMostGrid[key_words] : kMostCluster[key_words];
+  g.L = std::max(256, std::min(most, ((int)L + 31) / 32 * 32));
+  g.Lin = g.L;
+  g.entropy = entropy ? 1 : 0;
+  g.logB = 4;  // buckets of four slots, at most three quarters full
+  while (3 * (4 << g.logB) < 4 * g.L) ++g.logB;
+  return g;
+}
+
+// The most dynamic shared memory that a launch of a kernel takes, over its shapes.
+template <class KT>
+unsigned int most_bytes(bool grid, bool reverse) {
+  constexpr int kw = sizeof(KT) / 8;
+  unsigned int most = 0;
+  for (int ctas = 1; ctas <= (grid ? 1 : kMaxC); ctas *= 2)
+    most = std::max(most, res_layout<KT>(shape(ctas, grid, grid ? kMostGrid[kw] : kMostCluster[kw], true, kw), reverse).bytes);
+  return most;
+}
+
 // Launch configuration of a resident kernel; attr must outlive cfg.
 template <class Kernel, class KT>
 cudaError_t res_config(Kernel kernel, const KT&, int n_jobs, const ResGeom& g, bool reverse, cudaStream_t st,
                        cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
-  const unsigned int smem = res_layout<KT>(g, reverse).bytes;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // The limit belongs to the function, not to the launch: it is the same for every
+  // launch, whatever another host thread launches in between.
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)most_bytes<KT>(g.grid != 0, reverse));
   if (e != cudaSuccess) return e;
   if (!g.grid && g.ctas > 8) {  // a cluster of 16 is above the portable size
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1643,7 +1672,7 @@ cudaError_t res_config(Kernel kernel, const KT&, int n_jobs, const ResGeom& g, b
   }
   cfg->gridDim = dim3((unsigned int)(n_jobs * g.ctas));
   cfg->blockDim = dim3(kT);
-  cfg->dynamicSmemBytes = smem;
+  cfg->dynamicSmemBytes = res_layout<KT>(g, reverse).bytes;
   cfg->stream = st;
   if (g.grid) {
     attr->id = cudaLaunchAttributeCooperative;
@@ -1671,23 +1700,6 @@ cudaError_t res_launch(Kernel kernel, const ResJob<KT>& one, const ResJob<KT>* m
     if (e != cudaSuccess) return e;
   }
   return cudaLaunchKernelEx(&cfg, kernel, one, many, g, net);
-}
-
-// Entries a CTA holds at most: what fits its shared memory in either kernel
-// (inside a cluster the inboxes lie there too).
-constexpr int kMostCluster[3] = {0, 2048, 1792}, kMostGrid[3] = {0, 5632, 4352};
-
-ResGeom shape(int ctas, bool grid, double L, bool entropy, int key_words) {
-  ResGeom g{};
-  g.ctas = ctas;
-  g.grid = grid ? 1 : 0;
-  const int most = grid ? kMostGrid[key_words] : kMostCluster[key_words];
-  g.L = std::max(256, std::min(most, ((int)L + 31) / 32 * 32));
-  g.Lin = g.L;
-  g.entropy = entropy ? 1 : 0;
-  g.logB = 4;  // buckets of four slots, at most three quarters full
-  while (3 * (4 << g.logB) < 4 * g.L) ++g.logB;
-  return g;
 }
 
 template <class KT>

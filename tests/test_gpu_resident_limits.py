@@ -58,3 +58,27 @@ def test_reverse_meets_a_cut_larger_than_the_inboxes(torch_cuda, n_cut):
     ctx = context(p)
     assert_gradient(ctx.gradient(), p)
     assert ctx.stats()["cut"] >= (1 << 20) - n_cut
+
+
+def test_problems_of_several_sizes_in_several_threads(torch_cuda):
+    # Launches of one kernel with more and with less shared memory, from threads of their own.
+    import threading
+    big = dataclasses.replace(synth.fig3_problem().prefix(3), n_max=8000, n_cut=5000)
+    small = synth.make_problem(77, 9, 3, 3, 0.08).prefix(3)
+    errors = []
+
+    def work(p, runs):
+        try:
+            with torch_cuda.cuda.stream(torch_cuda.cuda.Stream()):
+                c = context(p)
+                for _ in range(runs):
+                    c.apply()
+        except Exception as e:  # the thread's failure is the test's
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(p, 2000)) for p in (big, small, small, big)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
