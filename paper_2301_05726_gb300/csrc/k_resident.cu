@@ -1639,7 +1639,8 @@ ResGeom shape(int ctas, bool grid, double L, bool entropy, int key_words) {
   g.ctas = ctas;
   g.grid = grid ? 1 : 0;
   const int most = grid ? kMostGrid[key_words] : kMostCluster[key_words];
-  g.L = std::max(256, std::min(most, ((int)L + 31) / 32 * 32));
+  // (the sector of an uncut problem can be any size: clamped before it is an int)
+  g.L = std::max(256, std::min(most, ((int)std::min(L, (double)most) + 31) / 32 * 32));
   g.Lin = g.L;
   g.entropy = entropy ? 1 : 0;
   g.logB = 4;  // buckets of four slots, at most three quarters full

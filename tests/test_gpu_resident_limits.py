@@ -24,10 +24,10 @@ def torch_cuda():
     return torch
 
 
-def doubling(n_factors, extra=()):
-    """Singles of distinct electrons into distinct orbitals of 20, so that every factor doubles the
-    table (2^20 determinants after all of them), then the rows of extra."""
-    n, half = 20, 10
+def doubling(n_factors, extra=(), n=20):
+    """Singles of distinct electrons into distinct orbitals, half of them filled, so that every factor
+    doubles the table, then the rows of extra."""
+    half = n // 2
     rng = np.random.default_rng(5)
     h, g = synth.make_integrals(rng, n)
     rows = [(2 * i + s, -1, 2 * (i + half) + s, -1) for s in (0, 1) for i in range(half)][:n_factors]
@@ -82,3 +82,14 @@ def test_problems_of_several_sizes_in_several_threads(torch_cuda):
     for t in threads:
         t.join()
     assert not errors, errors[0]
+
+
+def test_the_whole_gpu_serves_a_sector_of_any_size(torch_cuda):
+    # 3.6e17 determinants in the sector: the room is the GPU's, not the sector's.
+    p = doubling(17, n=32)
+    ctx, general = context(p), context(p, rebuild_test_regions=1)
+    for c in (ctx, general):
+        c.apply()
+    assert ctx.stats()["n_det"] == 1 << 17 and ctx.stats()["forward_launches"] == 1
+    for x, y in zip(ctx.wavefunction(), general.wavefunction()):
+        assert np.array_equal(x, y)
