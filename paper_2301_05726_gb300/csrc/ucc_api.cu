@@ -958,8 +958,11 @@ ucc_status run_factors(ucc_ctx* c, TableSet& s, double eps, bool record, int k0,
   UCC_TRY(resident_forward<KT>(c, s, eps, record, &k, k1));
   if (k == k1) return UCC_OK;
   UCC_TRY(ensure_hash<KT>(c, s));
-  if (k > k0) {
-    Counters known = *s.h_cnt;  // room for the next factor, as after every stop
+  // Room for the next factor, as after every stop.  A table that a resident pass
+  // of the segment before this one left needs it too: that pass leaves no more
+  // room than it needs itself.
+  if (k > k0 || 2 * s.h_cnt->n_tail > s.cur.cap_n || 8 * s.h_cnt->n_tail > 3 * s.cur.n_slots) {
+    Counters known = *s.h_cnt;
     UCC_TRY(ensure_room_known<KT>(c, s, record, &known));
     *s.h_cnt = known;
   }

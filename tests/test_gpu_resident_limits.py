@@ -93,3 +93,12 @@ def test_the_whole_gpu_serves_a_sector_of_any_size(torch_cuda):
     assert ctx.stats()["n_det"] == 1 << 17 and ctx.stats()["forward_launches"] == 1
     for x, y in zip(ctx.wavefunction(), general.wavefunction()):
         assert np.array_equal(x, y)
+
+
+def test_a_segment_that_starts_without_room(torch_cuda):
+    # 2^19 determinants at the end of a resident segment; the next one's only factor
+    # doubles them, past the resident room and past the table's capacity.
+    p = doubling(20)
+    ctx = context(p, checkpoint_stride=19)
+    assert_gradient(ctx.gradient(), p, checkpoint_stride=19)
+    assert ctx.stats()["n_det"] == 1 << 20
