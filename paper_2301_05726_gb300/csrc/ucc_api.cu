@@ -857,16 +857,28 @@ ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, const ResGeom& g, d
 
 // Tape for a resident forward pass that holds h.tape_n records: room for the
 // records of a few full tables (the launch stops when half of that is left),
-// and twice what there is (few launches) unless that passes the call's budget.
+// and twice what there is (few launches) where that can be had.  A tape that
+// cannot be had, within the call's budget, is left as it was.
 ucc_status resident_tape(ucc_ctx* c, const Counters& h, const ResGeom& g) {
   const unsigned long long most =
       std::min(most_entries(c), (unsigned long long)g.L * (unsigned long long)g.ctas);
   const unsigned long long need = h.tape_n + 12ull * most + (1ull << 12);
   if (c->tape_cap >= need && c->tape_cap >= 2ull * h.tape_n) return UCC_OK;
-  if (ensure_tape(c, std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
-  c->tape_over_budget = false;
-  cudaGetLastError();
-  return ensure_tape(c, need);
+  auto grow = [&](unsigned long long records) -> ucc_status {
+    const unsigned long long pages = (records + kTapePageRecs - 1) / kTapePageRecs;
+    if (c->tape_budget && pages * kTapePageRecs * c->tape_rec_bytes() > c->tape_budget)
+      return fail(UCC_ECAPACITY, "kill tape over its memory budget");
+    const size_t had = c->t_pages.size();
+    const ucc_status s = ensure_tape(c, records);
+    while (s != UCC_OK && c->t_pages.size() > had) {
+      dfree(c->t_pages.back());
+      c->t_pages.pop_back();
+      c->tape_cap -= kTapePageRecs;
+    }
+    return s;
+  };
+  if (grow(std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
+  return c->tape_cap >= need ? UCC_OK : grow(need);
 }
 
 // What a resident forward launch left in the job's counters (its host mirror).
@@ -888,7 +900,13 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
     const unsigned long long live = before.n_tail - before.n_dead;
     if (!res_room(live, g)) return UCC_OK;
     UCC_TRY(resident_net<KT>(c, g, &net));
-    if (record) UCC_TRY(resident_tape(c, before, g));
+    if (record) {
+      // A launch per factor needs tape for its next steps, not for full tables: it
+      // takes over where there is less.
+      const ucc_status t = resident_tape(c, before, g);
+      if (t == UCC_ECAPACITY || t == UCC_ENOMEM) return UCC_OK;
+      UCC_TRY(t);
+    }
     CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
     CUDA_TRY(launch_res_forward<KT>(resident_job<KT>(c, s, g, eps, *k, k1), nullptr, 1, g, net, record ? 1 : 0,
                                     c->stream));

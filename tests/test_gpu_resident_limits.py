@@ -102,3 +102,17 @@ def test_a_segment_that_starts_without_room(torch_cuda):
     ctx = context(p, checkpoint_stride=19)
     assert_gradient(ctx.gradient(), p, checkpoint_stride=19)
     assert ctx.stats()["n_det"] == 1 << 20
+
+
+@pytest.mark.parametrize("options", [dict(checkpoint_stride=100, tape_budget_mb=100), dict(tape_budget_mb=48)])
+def test_a_tape_that_fits_the_launches_but_not_full_tables(torch_cuda, options):
+    # Some 250,000 records in all, 140,000 in a segment (a page of 24 MiB); a resident
+    # pass over a table of this size wants ten times as many at once.
+    p = synth.make_problem(77, 15, 4, 4, 0.02, eps=1e-6).prefix(400)
+    ctx, general = context(p, **options), context(p, rebuild_test_regions=1, **options)
+    E, g = ctx.gradient()
+    Er, gr = general.gradient()
+    assert abs(E - Er) <= E_TOL and np.max(np.abs(g - gr)) <= G_TOL
+    st, sg = ctx.stats(), general.stats()
+    for x in ("tape_entries", "created", "dropped_old", "recompute_rotations"):
+        assert st[x] == sg[x], x
