@@ -646,6 +646,60 @@ ucc_status resident_net(ucc_ctx* c, const ResGeom& g, ResNet<KT>* net) {
   return UCC_OK;
 }
 
+// Tape for a resident forward pass that holds h.tape_n records: room for the
+// records of a few full tables (the launch stops when half of that is left),
+// and twice what there is (few launches) where that can be had.  A tape that
+// cannot be had, within the call's budget, is left as it was.
+ucc_status resident_tape(ucc_ctx* c, const Counters& h, const ResGeom& g) {
+  const unsigned long long most =
+      std::min(most_entries(c), (unsigned long long)g.L * (unsigned long long)g.ctas);
+  const unsigned long long need = h.tape_n + 12ull * most + (1ull << 12);
+  if (c->tape_cap >= need && c->tape_cap >= 2ull * h.tape_n) return UCC_OK;
+  auto grow = [&](unsigned long long records) -> ucc_status {
+    const unsigned long long pages = (records + kTapePageRecs - 1) / kTapePageRecs;
+    if (c->tape_budget && pages * kTapePageRecs * c->tape_rec_bytes() > c->tape_budget)
+      return fail(UCC_ECAPACITY, "kill tape over its memory budget");
+    const size_t had = c->t_pages.size();
+    const ucc_status s = ensure_tape(c, records);
+    while (s != UCC_OK && c->t_pages.size() > had) {
+      dfree(c->t_pages.back());
+      c->t_pages.pop_back();
+      c->tape_cap -= kTapePageRecs;
+    }
+    return s;
+  };
+  if (grow(std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
+  return c->tape_cap >= need ? UCC_OK : grow(need);
+}
+
+// What a resident run that starts with `live` determinants in table s needs before
+// its first factor (record: in a gradient): tape, inboxes, and room in the table
+// for what it may write back.  *ready = false: not all of that can be had.  Then no memory is
+// kept for it: a launch per factor, which runs instead, needs little at first.
+// The contents of s and of the tape are lost.
+template <class KT>
+ucc_status resident_prepare(ucc_ctx* c, TableSet& s, unsigned long long live, bool record, bool* ready) {
+  *ready = false;
+  ResGeom g{};
+  if (c->K == 0 || !resident_shape(c, &g) || !res_room(live, g)) return UCC_OK;
+  const unsigned long long cap = resident_cap(c, g);
+  ResNet<KT> net{};
+  ucc_status r = record ? resident_tape(c, Counters{}, g) : UCC_OK;
+  if (r == UCC_OK) r = resident_net<KT>(c, g, &net);
+  if (r == UCC_OK && s.cur.cap_n < cap) r = s.cur.allocate(cap, slots_for(cap));
+  if (r == UCC_ENOMEM) {
+    s.cur.release();
+    dfree(c->d_res_key);
+    dfree(c->d_res_val);
+    c->res_slots = 0;
+    release_tape(c);
+  } else if (r != UCC_ECAPACITY) {  // (a tape over the call's budget)
+    UCC_TRY(r);
+    *ready = true;
+  }
+  return UCC_OK;
+}
+
 template <class KT>
 KT reference_key(const ucc_ctx* c) {
   KT hf = KeyOps<KT>::zero();
@@ -699,12 +753,10 @@ ucc_status reset_tape(ucc_ctx* c, TableSet& s, int k0) {
 // Load a snapshot into table s (its previous contents are discarded).
 template <class KT>
 ucc_status load_snapshot(ucc_ctx* c, TableSet& s, const Snapshot& snap) {
-  unsigned long long cap = std::max<unsigned long long>(4 * snap.n, 1 << 12);
-  {
-    ResGeom g{};
-    if (resident_shape(c, &g)) cap = std::max(cap, resident_cap(c, g));
-  }
+  const unsigned long long cap = std::max<unsigned long long>(4 * snap.n, 1 << 12);
   if (cap >= kMaxEntries) return fail(UCC_ECAPACITY, "snapshot too large for one table");
+  bool resident = false;
+  UCC_TRY(resident_prepare<KT>(c, s, snap.n, true, &resident));
   if (s.cur.cap_n < cap) UCC_TRY(s.cur.allocate(cap, slots_for(cap)));
   s.hash_valid = true;
   CUDA_TRY(cudaMemsetAsync(s.d_cnt, 0, sizeof(Counters), c->stream));
@@ -855,32 +907,6 @@ ResJob<KT> resident_job(const ucc_ctx* c, const TableSet& s, const ResGeom& g, d
   return j;
 }
 
-// Tape for a resident forward pass that holds h.tape_n records: room for the
-// records of a few full tables (the launch stops when half of that is left),
-// and twice what there is (few launches) where that can be had.  A tape that
-// cannot be had, within the call's budget, is left as it was.
-ucc_status resident_tape(ucc_ctx* c, const Counters& h, const ResGeom& g) {
-  const unsigned long long most =
-      std::min(most_entries(c), (unsigned long long)g.L * (unsigned long long)g.ctas);
-  const unsigned long long need = h.tape_n + 12ull * most + (1ull << 12);
-  if (c->tape_cap >= need && c->tape_cap >= 2ull * h.tape_n) return UCC_OK;
-  auto grow = [&](unsigned long long records) -> ucc_status {
-    const unsigned long long pages = (records + kTapePageRecs - 1) / kTapePageRecs;
-    if (c->tape_budget && pages * kTapePageRecs * c->tape_rec_bytes() > c->tape_budget)
-      return fail(UCC_ECAPACITY, "kill tape over its memory budget");
-    const size_t had = c->t_pages.size();
-    const ucc_status s = ensure_tape(c, records);
-    while (s != UCC_OK && c->t_pages.size() > had) {
-      dfree(c->t_pages.back());
-      c->t_pages.pop_back();
-      c->tape_cap -= kTapePageRecs;
-    }
-    return s;
-  };
-  if (grow(std::max(need, 2ull * h.tape_n)) == UCC_OK) return UCC_OK;
-  return c->tape_cap >= need ? UCC_OK : grow(need);
-}
-
 // What a resident forward launch left in the job's counters (its host mirror).
 void resident_account(ucc_ctx* c, const Counters& h) {
   c->cut_total += (long long)h.res_cut;
@@ -899,7 +925,10 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
     const Counters before = *s.h_cnt;
     const unsigned long long live = before.n_tail - before.n_dead;
     if (!res_room(live, g)) return UCC_OK;
-    UCC_TRY(resident_net<KT>(c, g, &net));
+    // (without memory for the inboxes: a launch per factor, which needs none)
+    const ucc_status n = resident_net<KT>(c, g, &net);
+    if (n == UCC_ENOMEM) return UCC_OK;
+    UCC_TRY(n);
     if (record) {
       // A launch per factor needs tape for its next steps, not for full tables: it
       // takes over where there is less.
@@ -945,7 +974,9 @@ ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int k1, bool* done)
   if (!resident_shape(c, &g) || s.cur.cap_n < resident_cap(c, g)) return UCC_OK;
   if (!res_room(s.h_cnt->n_tail - s.h_cnt->n_dead, g)) return UCC_OK;
   ResNet<KT> net{};
-  UCC_TRY(resident_net<KT>(c, g, &net));
+  const ucc_status n = resident_net<KT>(c, g, &net);
+  if (n == UCC_ENOMEM) return UCC_OK;
+  UCC_TRY(n);
   CUDA_TRY(cudaEventRecord(c->kev[0], c->stream));
   CUDA_TRY(launch_res_reverse<KT>(resident_job<KT>(c, s, g, 0.0, k0, k1), nullptr, 1, g, net, c->stream));
   CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
@@ -1096,10 +1127,10 @@ int segment_stride(const ucc_ctx* c) {
 
 // The reference state in table s, sized and (not) hashed for the path that runs first.
 template <class KT>
-ucc_status reset_for_run(ucc_ctx* c, TableSet& s) {
-  ResGeom g{};
-  const bool resident = c->K > 0 && resident_shape(c, &g);
-  return reset_table<KT>(c, s, !resident, resident ? resident_cap(c, g) : 0ull);
+ucc_status reset_for_run(ucc_ctx* c, TableSet& s, bool record) {
+  bool resident = false;
+  UCC_TRY(resident_prepare<KT>(c, s, 1, record, &resident));
+  return reset_table<KT>(c, s, !resident);
 }
 
 template <class KT>
@@ -1109,7 +1140,7 @@ ucc_status run_forward(ucc_ctx* c, double eps, bool record) {
   c->cut_total = 0;
   c->entropy_on = !record && c->opt.record_entropy != 0;
   c->have_entropy = false;
-  UCC_TRY(reset_for_run<KT>(c, s));
+  UCC_TRY(reset_for_run<KT>(c, s, record));
   CUDA_TRY(cudaEventRecord(c->ev[0], c->stream));
   if (!record) {
     UCC_TRY(run_factors<KT>(c, s, eps, false, 0, c->K));
@@ -1450,7 +1481,7 @@ ucc_status run_gradient_once(ucc_ctx* c, double eps, double* E, double* grad_out
       TableSet& from = c->ts[c->main];
       TableSet& work = c->ts[1 - c->main];
       if (j == 0) {
-        UCC_TRY(reset_for_run<KT>(c, work));
+        UCC_TRY(reset_for_run<KT>(c, work, true));
       } else {
         UCC_TRY(load_snapshot<KT>(c, work, c->snaps[j]));
       }

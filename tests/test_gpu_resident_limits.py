@@ -116,3 +116,30 @@ def test_a_tape_that_fits_the_launches_but_not_full_tables(torch_cuda, options):
     st, sg = ctx.stats(), general.stats()
     for x in ("tape_entries", "created", "dropped_old", "recompute_rotations"):
         assert st[x] == sg[x], x
+
+
+@pytest.mark.parametrize("left_mb", [44, 84, 120])
+def test_less_memory_than_a_resident_pass_wants(torch_cuda, left_mb):
+    # A resident gradient over this sector wants a table of 66 MB, for what it may
+    # write back, inboxes of 41 MB and 240 MB of tape; 14,841 determinants
+    # take some 5 MB, and a launch per factor one page of tape, 24 MiB.
+    torch = torch_cuda
+    p = synth.make_problem(77, 15, 4, 4, 0.05).prefix(60)
+    options = dict(energy_route=1)  # the bucketed energy's buffers have their own fallback
+    for more in (dict(), dict(rebuild_test_regions=1)):
+        context(p, **options, **more).gradient()  # every kernel is loaded
+    ctx = context(p, **options)
+    hold = []
+    try:
+        torch.cuda.synchronize()
+        for step in (1 << 30, 1 << 24, 1 << 21):
+            while torch.cuda.mem_get_info()[0] > (left_mb << 20) + step:
+                n = (torch.cuda.mem_get_info()[0] - (left_mb << 20)) // step * step
+                hold.append(torch.empty(n, dtype=torch.uint8, device="cuda"))
+        ctx.apply()
+        E, g = ctx.gradient()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert ctx.stats()["forward_launches"] >= p.n_exc  # no resident pass
+    assert_gradient((E, g), p, **options)
