@@ -94,24 +94,31 @@ typedef struct {
                            largest |c| (ties: smaller key).  0 = off. */
   int64_t max_entries;  /* hard cap on stored determinants, 0 = device memory */
   int32_t probe_width;  /* lanes per hash probe: 1, 2, 4 or 8; 0 = autotuned.
-                           Tables that fit a thread-block cluster's shared
-                           memory run resident in it, a whole run of factors
-                           per launch, unless probe_width, max_entries or
-                           rebuild_test_regions is set (their results are the
-                           same) */
+                           Tables that fit shared memory run resident, a whole
+                           run of factors per launch, unless probe_width,
+                           max_entries or rebuild_test_regions is set (their
+                           results are the same): up to some 25,000
+                           determinants in one thread-block cluster, up to some
+                           700,000 in a cooperative launch over the whole GPU */
   int32_t checkpoint_stride; /* gradient: factors between snapshots of psi; 0 =
                                 one segment while the kill tape fits its
                                 budget, else ceil(sqrt(K)) */
   int32_t tape_budget_mb;    /* kill-tape budget in MiB; 0 = 60% of free memory */
   int32_t record_entropy;    /* ucc_apply records Eq. 6 after every factor */
-  int32_t batch_wait_ms;     /* ucc_batch_run: bound of one grid-barrier wait of
-                                its persistent launches, in ms; 0 = 2000.  Read
-                                from the first job. */
+  int32_t batch_wait_ms;     /* bound of one grid-barrier wait, in ms; 0 = 2000.
+                                ucc_batch_run: of its persistent launches, read
+                                from the first job (UCC_ETIMEOUT when it runs
+                                out).  Other calls: of whole-GPU resident
+                                launches; when it runs out before the launch
+                                writes its table back (work on another stream
+                                held SMs that long), the factors run with a
+                                launch each, else UCC_ETIMEOUT */
   int32_t batch_test_skip_block; /* test only: block (1-based) of the batch's
                                     persistent forward launch that leaves
                                     before its first grid barrier, so that the
                                     others' bounded waits run out and the call
-                                    returns UCC_ETIMEOUT; 0 = none */
+                                    returns UCC_ETIMEOUT, or (2 and above) of
+                                    whole-GPU resident launches; 0 = none */
   int32_t batch_tiles;       /* ucc_batch_run: 32-entry tiles a warp takes per
                                 visit of a job (1, 2, 4 or 8); 0 = autotuned.
                                 Read from the first job. */

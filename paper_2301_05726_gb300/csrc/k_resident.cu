@@ -31,7 +31,8 @@
 // Inside a cluster messages are remote shared-memory stores and the barrier is
 // the cluster's; across the GPU the inboxes lie in L2 and the barrier is one
 // 64-bit word whose arrivals carry the sums (a cooperative launch, every wait
-// bounded).
+// bounded: one that runs out ends the launch, and the host runs the same factors
+// with a launch each).
 //
 // What bounds it: latency, of the barrier (0.8 us in a cluster of sixteen, 2 us
 // across the GPU), of a message (0.5 and 1 us) and of the block's own phases.
@@ -72,7 +73,6 @@ constexpr int kWinShift = 44;  // ... of 2^44 in |c|'s bits, 256 an octave
 constexpr int kOffRing = 256;  // tape offsets held at a time
 constexpr int kMaxC = 16;      // CTAs of a cluster
 constexpr int kMaxG = 240;     // CTAs of a grid (arrivals are counted in 8 bits)
-constexpr unsigned long long kWaitNs = 2000000000ull;  // bound of one grid barrier
 
 // What a barrier sums over the CTAs, in one 64-bit word: arrivals (8 bits),
 // CTAs that must abort (8), CTAs that see the tape running low (8), linked
@@ -234,6 +234,7 @@ struct GridNet {
   double* ina;
   unsigned long long* inb;
   unsigned int C, rank, Lin, epoch;
+  unsigned long long wait_ns;
 
   __device__ __forceinline__ unsigned int* counter(int buf, int kind, unsigned int owner) const {
     return &ctl->count[buf][kind][owner][0];
@@ -268,7 +269,7 @@ struct GridNet {
         for (;;) {
           v = *((volatile unsigned long long*)w);
           if ((v & 0xFFull) == (unsigned long long)C) break;
-          if ((++spins & 255u) == 0u && ns_now() - t0 > kWaitNs) {
+          if ((++spins & 255u) == 0u && ns_now() - t0 > wait_ns) {
             raise_error(cnt, ERR_TIMEOUT);
             v = pack_word(true, false, 0u, 0u);
             break;
@@ -370,6 +371,7 @@ __device__ __forceinline__ GridNet<KT> make_net(GridNet<KT>*, unsigned char*, co
   n.rank = blockIdx.x;
   n.Lin = (unsigned int)g.Lin;
   n.epoch = 0u;
+  n.wait_ns = r.wait_ns;
   return n;
 }
 
@@ -620,7 +622,10 @@ __device__ __forceinline__ bool res_load(const ResView<KT>& v, Net& net, const T
 template <class KT>
 __device__ __forceinline__ void res_store(const ResView<KT>& v, const TableT<KT>& t, unsigned int n) {
   __shared__ unsigned long long s_base;
-  if (threadIdx.x == 0) s_base = atomicAdd(&t.cnt->res_n, (unsigned long long)n);
+  if (threadIdx.x == 0) {
+    atomicAdd(&t.cnt->res_stored, 1u);
+    s_base = atomicAdd(&t.cnt->res_n, (unsigned long long)n);
+  }
   __syncthreads();
   const unsigned long long base = s_base;
   for (unsigned int i = threadIdx.x; i < n; i += kT) {
@@ -1075,6 +1080,7 @@ __device__ __forceinline__ void res_finish(Counters* c, unsigned long long* off,
     c->n_scan = m;
     c->n_dead = 0ull;
     c->res_n = 0ull;
+    c->res_stored = 0u;
     c->stop_k = -1;
   }
 }
@@ -1092,6 +1098,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
   __shared__ int s_full, s_low;
   __shared__ unsigned long long s_tbase;
   __shared__ NetShared s_net;
+  if (Net::kGrid && blockIdx.x != 0u && blockIdx.x + 1u == rnet.skip_block) return;
   const ResLayout lo = res_layout<KT>(g, false);
   const ResJob<KT> job = many ? many[blockIdx.x / (unsigned int)g.ctas] : one;
   const ResView<KT> v = res_view<KT>(res_smem, lo, g, false);
@@ -1377,7 +1384,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
   }
   // What happened in the last step is flagged here (nothing else is in flight).
   if (status != RES_ABORT && word_abort(net_sync(net, pack_word(s_full != 0, false, 0u, 0u), cnt))) status = RES_ABORT;
-  const bool store = status != RES_ABORT && k > job.k0;
+  bool store = status != RES_ABORT && k > job.k0;
   if (store) {
     if (ent && k > job.k0) add_sum(&job.t.entropy[k - 1], dS_due);
     const unsigned int kept = res_squeeze(v, n_scan);
@@ -1391,8 +1398,11 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
       if (so) atomicAdd(&cnt->dropped_old, so);
     }
     if (tid == 0) atomicAdd(&cnt->scanned, scanned);
-    net_sync(net, pack_word(false, false, 0u, 0u), cnt);  // every CTA's entries and counts are there
-    if (net.rank == 0u)
+    // every CTA's entries and counts are there, or a CTA gave up and never will be
+    if (word_abort(net_sync(net, pack_word(false, false, 0u, 0u), cnt))) {
+      store = false;
+      status = RES_ABORT;
+    } else if (net.rank == 0u)
       res_finish(cnt, RECORD ? job.tape.off : nullptr, job.t.entropy, job.k0, k, res_smem);
   }
   if (net.rank == 0u && tid == 0) {
@@ -1423,6 +1433,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
   __shared__ int s_full;
   __shared__ unsigned long long s_off[kOffRing + 1];
   __shared__ NetShared s_net;
+  if (Net::kGrid && blockIdx.x != 0u && blockIdx.x + 1u == rnet.skip_block) return;
   const ResLayout lo = res_layout<KT>(g, true);
   const ResJob<KT> job = many ? many[blockIdx.x / (unsigned int)g.ctas] : one;
   const ResView<KT> v = res_view<KT>(res_smem, lo, g, true);
@@ -1619,8 +1630,11 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
     const unsigned long long sp = warp_sum_u64(pairs);
     if (lane == 0 && sp) atomicAdd(&cnt->rev_pairs, sp);
     if (tid == 0) atomicAdd(&cnt->rev_scanned, scanned);
-    net_sync(net, pack_word(false, false, 0u, 0u), cnt);  // every CTA's entries and counts are there
-    if (net.rank == 0u) res_finish(cnt, nullptr, nullptr, job.k0, job.k0, res_smem);
+    // (as in the forward pass)
+    if (word_abort(net_sync(net, pack_word(false, false, 0u, 0u), cnt)))
+      status = RES_ABORT;
+    else if (net.rank == 0u)
+      res_finish(cnt, nullptr, nullptr, job.k0, job.k0, res_smem);
   }
   if (net.rank == 0u && tid == 0) {
     cnt->res_status = status;

@@ -202,6 +202,7 @@ struct ucc_ctx {
   unsigned long long* d_res_key = nullptr;
   unsigned long long* d_res_val = nullptr;
   size_t res_slots = 0;
+  bool res_gave_up = false;  // a resident launch of this call timed out: launches per factor for the rest of it
   SelectState* d_sel = nullptr;
   void* d_cand = nullptr;  // SelectCandT<KT>[kSelectCandCap]: candidates of the cut's last selection passes
   double* d_entropy = nullptr;  // [K] Eq. 6 after each factor of the last apply
@@ -611,6 +612,7 @@ unsigned long long most_entries(const ucc_ctx* c) {
 // fixed probe width, an entry cap that its chunks check, the region-build
 // test hook).
 bool resident_shape(const ucc_ctx* c, ResGeom* g) {
+  if (c->res_gave_up) return false;
   if (c->opt.rebuild_test_regions != 0 || c->opt.probe_width != 0 || c->opt.max_entries > 0) return false;
   const ResLimits lim = res_limits(c->kw);
   const unsigned long long most = most_entries(c);
@@ -643,6 +645,8 @@ ucc_status resident_net(ucc_ctx* c, const ResGeom& g, ResNet<KT>* net) {
   net->key = reinterpret_cast<KT*>(c->d_res_key);
   net->a = reinterpret_cast<double*>(c->d_res_val);
   net->b = c->d_res_val + c->res_slots;
+  net->wait_ns = c->opt.batch_wait_ms > 0 ? 1000000ull * (unsigned long long)c->opt.batch_wait_ms : 2000000000ull;
+  net->skip_block = (unsigned int)c->opt.batch_test_skip_block;
   return UCC_OK;
 }
 
@@ -914,6 +918,21 @@ void resident_account(ucc_ctx* c, const Counters& h) {
   c->stats.peak_entries = std::max<long long>(c->stats.peak_entries, (long long)h.res_peak);
 }
 
+// The counters after a resident launch.  A wait that ran out before any CTA wrote
+// back left the table as it was, so the launch counts as given up (RES_ABORT);
+// one that ran out where the launch went on to its end is no error.
+ucc_status read_resident(ucc_ctx* c, TableSet& s) {
+  CUDA_TRY(cudaMemcpyAsync(s.h_cnt, s.d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(cudaStreamSynchronize(c->stream));
+  Counters& h = *s.h_cnt;
+  if (h.error == ERR_TIMEOUT && (h.res_status != RES_ABORT || h.res_stored == 0)) {
+    CUDA_TRY(cudaMemsetAsync(&s.d_cnt->error, 0, sizeof(int), c->stream));
+    h.error = 0;
+    c->res_gave_up = true;
+  }
+  return check_device_error(h);
+}
+
 // As many of the factors [*k, k1) as the shape holds, on table s, whose
 // counters the host mirror holds; *k moves to the first one left.
 template <class KT>
@@ -942,7 +961,7 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
     CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
     c->launches++;
     c->stats.forward_launches++;
-    UCC_TRY(read_counters(c, s));
+    UCC_TRY(read_resident(c, s));
     float ms = 0.f;
     CUDA_TRY(cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]));
     c->stats.forward_kernel_ms += ms;
@@ -982,7 +1001,7 @@ ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int k1, bool* done)
   CUDA_TRY(cudaEventRecord(c->kev[1], c->stream));
   c->launches++;
   c->stats.reverse_launches++;
-  UCC_TRY(read_counters(c, s));
+  UCC_TRY(read_resident(c, s));
   float ms = 0.f;
   CUDA_TRY(cudaEventElapsedTime(&ms, c->kev[0], c->kev[1]));
   c->stats.reverse_kernel_ms += ms;
@@ -1138,6 +1157,7 @@ ucc_status run_forward(ucc_ctx* c, double eps, bool record) {
   if (!(eps >= 0.0) || std::isinf(eps)) return fail(UCC_EINVAL, "eps must be finite and >= 0");
   TableSet& s = c->ts[c->main];
   c->cut_total = 0;
+  c->res_gave_up = false;
   c->entropy_on = !record && c->opt.record_entropy != 0;
   c->have_entropy = false;
   UCC_TRY(reset_for_run<KT>(c, s, record));

@@ -64,6 +64,7 @@ struct Counters {
   int res_status, res_k;
   unsigned long long res_cut, res_n;  // res_n: entries written back (0 between launches)
   unsigned int res_rebuilds, res_peak;
+  unsigned int res_stored;  // CTAs that have begun to write back (0 between launches)
 };
 
 // How a resident launch ended.
@@ -93,7 +94,7 @@ enum DeviceError : int {
   ERR_CONSISTENCY = 2,   // a state the algorithm excludes was observed
   ERR_TAPE_FULL = 4,     // kill tape capacity exceeded
   ERR_CAPACITY = 8,      // entry allocation past capacity
-  ERR_TIMEOUT = 16       // a resident launch's grid barrier gave up waiting
+  ERR_TIMEOUT = 16       // a whole-grid resident launch's barrier gave up waiting
 };
 
 // Everything a kernel needs to address the wavefunction table.
@@ -206,13 +207,17 @@ struct ResControl {
   unsigned long long cand_mag[512], cand_key[1024];
 };
 
-// ... and its inboxes, [2][ctas][Lin] each (null for clusters).
+// ... and its inboxes, [2][ctas][Lin] each (null for clusters), the bound of one
+// barrier's wait, and the test hook: this block (1-based; not the first, which
+// reports) leaves before its first barrier.
 template <class KT>
 struct ResNet {
   ResControl* ctl;
   KT* key;
   double* a;
   unsigned long long* b;
+  unsigned long long wait_ns;
+  unsigned int skip_block;
 };
 
 // Largest cluster, and CTAs of a whole-grid launch, that the current device

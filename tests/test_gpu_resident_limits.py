@@ -143,3 +143,33 @@ def test_less_memory_than_a_resident_pass_wants(torch_cuda, left_mb):
         torch.cuda.empty_cache()
     assert ctx.stats()["forward_launches"] >= p.n_exc  # no resident pass
     assert_gradient((E, g), p, **options)
+
+
+@pytest.mark.parametrize("wide", [False, True])
+def test_a_wait_that_runs_out(torch_cuda, wide):
+    # A block of every whole-GPU launch leaves before its first barrier (a test hook),
+    # so the others' waits run out after 50 ms: a launch per factor takes over.
+    p = (synth.make_problem(77, 34, 3, 3, 0.08, eps=1e-7).prefix(120) if wide
+         else synth.make_problem(77, 12, 4, 4, 0.08).prefix(120))
+    if wide:
+        p.n_max, p.n_cut = 24000, 15000
+    hook = dict(batch_wait_ms=50, batch_test_skip_block=2)
+    ctx, general = context(p, **hook), context(p, rebuild_test_regions=1)
+    for c in (ctx, general):
+        c.apply()
+    assert ctx.stats()["forward_launches"] > p.n_exc  # the one that gave up, and one per factor
+    for x, y in zip(ctx.wavefunction(), general.wavefunction()):
+        assert np.array_equal(x, y)
+    assert_gradient(ctx.gradient(), p)
+    assert_gradient(context(p, checkpoint_stride=25, **hook).gradient(), p)
+    entropies = []
+    for options in (hook, dict(rebuild_test_regions=1)):
+        c = context(p, record_entropy=1, **options)
+        c.apply()
+        entropies.append(c.entropy())
+    assert np.max(np.abs(entropies[0] - entropies[1])) <= 1e-10
+    ctx.set_options(batch_wait_ms=0, batch_test_skip_block=0)  # the same context runs resident again
+    ctx.apply()
+    assert ctx.stats()["forward_launches"] == 1
+    for x, y in zip(ctx.wavefunction(), general.wavefunction()):
+        assert np.array_equal(x, y)
