@@ -648,8 +648,10 @@ __host__ __device__ inline float largest_share(float most, int C) {
 }
 
 // Whether a CTA's dropped entries should leave: they are a third of its
-// entries, or an eighth where more than half of its room is taken (its room is
-// a quarter above the largest share of live ones, so what may still come fits).
+// entries, or an eighth where more than half of its room is taken.  Its room is a
+// quarter above the largest share of live ones, up to what its shared memory
+// holds; a step whose new entries do not fit beside the dropped ones has them
+// leave first.
 __device__ __forceinline__ bool res_crowded(unsigned int n, unsigned int dead, unsigned int L) {
   return dead > 64u ? 3u * dead > n || (2u * n > L && 8u * dead > n) : dead > 0u && 2u * n > L && 8u * dead > n;
 }
@@ -1146,7 +1148,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
   if (tid == 0 && !loaded) s_full = 1;
 
   int status = RES_DONE, k = job.k0;
-  unsigned int n_scan = min(s_tail, v.L);
+  unsigned int n_scan = min(s_tail, v.L), dead = 0u;  // dead: as the last step left it (block-uniform)
   unsigned int rot = 0, cre = 0, dnew = 0, dold = 0, rebuilds = 0, peak = 0;
   unsigned long long scanned = 0, cut_total = 0;
   // records that one step (and the stop after it) may need
@@ -1216,6 +1218,21 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
     Msg<KT> msg = net.template get<false>(buf, 0, min(tid, net.Lin - 1u));
     const unsigned int got = net.received(buf, 0);
     if (got > net.Lin) s_full = 1;
+    if (dead && n_scan + got > v.L) {
+      // No room beside the dropped entries for what the messages may create.
+      __syncthreads();  // (the queue's length is cleared)
+      if (tid == 0) scanned += n_scan;
+      n_scan = res_squeeze(v, n_scan);
+      if (tid == 0) {
+        s_tail = n_scan;
+        s_dead = 0u;
+      }
+      res_rehash(v, n_scan, cnt);
+      ++rebuilds;
+      res_scan(v, f, n_scan, &s_qn);  // the linked entries have moved
+      __syncthreads();
+      if (tid == 0) s_qn = 0u;
+    }
     for (unsigned int x = tid; x < min(got, net.Lin); x += kT) {
       if (x != tid) msg = net.template get<false>(buf, 0, x);
       const KT Z = msg.key;
@@ -1368,7 +1385,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
         ++rebuilds;
       }
     }
-    const unsigned int dead = s_dead;  // (block-uniform: written only in phase B)
+    dead = s_dead;  // (block-uniform: written only in phase B)
     if (res_crowded(n_scan, dead, v.L)) {
       const unsigned int kept = res_squeeze(v, n_scan);
       if (tid == 0) {
@@ -1376,6 +1393,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
         s_dead = 0u;
       }
       n_scan = linked_to = kept;
+      dead = 0u;
       res_rehash(v, kept, cnt);
       ++rebuilds;
     }
@@ -1583,6 +1601,23 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
         v.amps[i] = x0;
         v.lam[i] = l0;
         ++pairs;
+      }
+    }
+    if (n_scan + recs > v.L) {
+      // No room beside dropped entries for the records: they leave first.
+      __syncthreads();
+      const unsigned int dead = s_dead;
+      __syncthreads();  // (read by every thread before the records change it)
+      if (dead) {
+        const unsigned int kept = res_squeeze(v, n_scan);
+        if (tid == 0) {
+          s_tail = kept;
+          s_dead = 0u;
+          if (sweep) scanned += n_scan - kept;
+        }
+        n_scan = kept;
+        res_rehash(v, kept, cnt);
+        ++compactions;
       }
     }
     // The records of factor k - 1: a key that is still stored was dropped.

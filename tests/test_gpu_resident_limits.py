@@ -173,3 +173,38 @@ def test_a_wait_that_runs_out(torch_cuda, wide):
     assert ctx.stats()["forward_launches"] == 1
     for x, y in zip(ctx.wavefunction(), general.wavefunction()):
         assert np.array_equal(x, y)
+
+
+def test_dropped_entries_near_the_room(torch_cuda):
+    # 714,208 determinants, near the 760,000 that the GPU holds, then factors of angle
+    # pi/2: each moves some 5 % of them, so that what it leaves behind is dropped.
+    base = synth.make_problem(77, 24, 3, 3, 0.15, eps=1e-12)
+    p = dataclasses.replace(base.prefix(260), n_max=715_000, n_cut=705_000)
+    ctx = context(p)
+    ctx.apply()
+    keys = ctx.wavefunction()[0][::7]
+
+    def linked(row):
+        i, j, a, b = (int(x) for x in row)
+        occ, vir = np.uint64((1 << i) | (1 << j)), np.uint64((1 << a) | (1 << b))
+        x = keys & (occ | vir)
+        return float(np.mean((x == occ) | (x == vir)))
+
+    rows = [r for r in base.exc[260:] if r[1] >= 0]
+    rows = np.array([r for r in rows if 0.045 < linked(r) < 0.06][:40], dtype=np.int32)
+    assert len(rows) == 40
+    p = dataclasses.replace(p, exc=np.concatenate([p.exc, rows]),
+                            theta=np.concatenate([p.theta, np.full(len(rows), np.pi / 2)]))
+    ctx, general = context(p), context(p, rebuild_test_regions=1)
+    for c in (ctx, general):
+        c.apply()
+    st, sg = ctx.stats(), general.stats()
+    for x in ("n_det", "rotations", "created", "dropped_new", "dropped_old", "cut"):
+        assert st[x] == sg[x], x
+    assert st["dropped_old"] > 500_000 and st["forward_launches"] == 1
+    for x, y in zip(ctx.wavefunction(), general.wavefunction()):
+        assert np.array_equal(x, y)
+    ctx.gradient()  # (more tape may be needed on the way: a second launch)
+    E, g = ctx.gradient()
+    assert_gradient((E, g), p)
+    assert ctx.stats()["forward_launches"] == 1 and ctx.stats()["reverse_launches"] == 1
