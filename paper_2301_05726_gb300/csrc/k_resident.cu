@@ -649,9 +649,11 @@ __host__ __device__ inline float largest_share(float most, int C) {
 
 // Whether a CTA's dropped entries should leave: they are a third of its
 // entries, or an eighth where more than half of its room is taken.  Its room is a
-// quarter above the largest share of live ones, up to what its shared memory
-// holds; a step whose new entries do not fit beside the dropped ones has them
-// leave first.
+// quarter above the largest share of live ones, so what may still come fits: always
+// in a cluster, and across the GPU up to what the shared memory holds.  Above that
+// (some 600,000 one-word entries) a step whose new entries do not fit beside the
+// dropped ones has them leave first; that code in the cluster's kernels, where
+// nothing reaches it, costs the gradient at 72 spin-orbitals 3 %.
 __device__ __forceinline__ bool res_crowded(unsigned int n, unsigned int dead, unsigned int L) {
   return dead > 64u ? 3u * dead > n || (2u * n > L && 8u * dead > n) : dead > 0u && 2u * n > L && 8u * dead > n;
 }
@@ -1218,7 +1220,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
     Msg<KT> msg = net.template get<false>(buf, 0, min(tid, net.Lin - 1u));
     const unsigned int got = net.received(buf, 0);
     if (got > net.Lin) s_full = 1;
-    if (dead && n_scan + got > v.L) {
+    if (Net::kGrid && dead && n_scan + got > v.L) {
       // No room beside the dropped entries for what the messages may create.
       __syncthreads();  // (the queue's length is cleared)
       if (tid == 0) scanned += n_scan;
@@ -1603,7 +1605,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
         ++pairs;
       }
     }
-    if (n_scan + recs > v.L) {
+    if (Net::kGrid && n_scan + recs > v.L) {
       // No room beside dropped entries for the records: they leave first.
       __syncthreads();
       const unsigned int dead = s_dead;
