@@ -649,13 +649,16 @@ __host__ __device__ inline float largest_share(float most, int C) {
 
 // Whether a CTA's dropped entries should leave: they are a third of its
 // entries, or an eighth where more than half of its room is taken.  Its room is a
-// quarter above the largest share of live ones, so what may still come fits: always
-// in a cluster, and across the GPU up to what the shared memory holds.  Above that
-// (some 600,000 one-word entries) a step whose new entries do not fit beside the
-// dropped ones has them leave first; that code in the cluster's kernels, where
-// nothing reaches it, costs the gradient at 72 spin-orbitals 3 %.
+// quarter above the largest share of live ones, so what may still come fits -- except
+// where its shared memory holds less than that quarter (from some 600,000 one-word
+// entries on the GPU): with the last ninth of the room taken they leave from 3 % on,
+// so that a step may add a ninth.  (An exact test in the step itself, on the messages
+// received, costs the energy at 24 spin-orbitals 0.4 % and, with two-word keys, the
+// gradient at 72 3 %.)
 __device__ __forceinline__ bool res_crowded(unsigned int n, unsigned int dead, unsigned int L) {
-  return dead > 64u ? 3u * dead > n || (2u * n > L && 8u * dead > n) : dead > 0u && 2u * n > L && 8u * dead > n;
+  if (dead == 0u) return false;
+  if (2u * n > L) return (9u * n > 8u * L ? 32u : 8u) * dead > n;
+  return dead > 64u && 3u * dead > n;
 }
 
 // Exclusive block prefix of one count per thread; *total in every thread.
@@ -1150,7 +1153,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
   if (tid == 0 && !loaded) s_full = 1;
 
   int status = RES_DONE, k = job.k0;
-  unsigned int n_scan = min(s_tail, v.L), dead = 0u;  // dead: as the last step left it (block-uniform)
+  unsigned int n_scan = min(s_tail, v.L);
   unsigned int rot = 0, cre = 0, dnew = 0, dold = 0, rebuilds = 0, peak = 0;
   unsigned long long scanned = 0, cut_total = 0;
   // records that one step (and the stop after it) may need
@@ -1220,21 +1223,6 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
     Msg<KT> msg = net.template get<false>(buf, 0, min(tid, net.Lin - 1u));
     const unsigned int got = net.received(buf, 0);
     if (got > net.Lin) s_full = 1;
-    if (Net::kGrid && dead && n_scan + got > v.L) {
-      // No room beside the dropped entries for what the messages may create.
-      __syncthreads();  // (the queue's length is cleared)
-      if (tid == 0) scanned += n_scan;
-      n_scan = res_squeeze(v, n_scan);
-      if (tid == 0) {
-        s_tail = n_scan;
-        s_dead = 0u;
-      }
-      res_rehash(v, n_scan, cnt);
-      ++rebuilds;
-      res_scan(v, f, n_scan, &s_qn);  // the linked entries have moved
-      __syncthreads();
-      if (tid == 0) s_qn = 0u;
-    }
     for (unsigned int x = tid; x < min(got, net.Lin); x += kT) {
       if (x != tid) msg = net.template get<false>(buf, 0, x);
       const KT Z = msg.key;
@@ -1387,7 +1375,7 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
         ++rebuilds;
       }
     }
-    dead = s_dead;  // (block-uniform: written only in phase B)
+    const unsigned int dead = s_dead;  // (block-uniform: written only in phase B)
     if (res_crowded(n_scan, dead, v.L)) {
       const unsigned int kept = res_squeeze(v, n_scan);
       if (tid == 0) {
@@ -1395,7 +1383,6 @@ __global__ void __launch_bounds__(kT, 1) k_res_forward(ResJob<KT> one, const Res
         s_dead = 0u;
       }
       n_scan = linked_to = kept;
-      dead = 0u;
       res_rehash(v, kept, cnt);
       ++rebuilds;
     }
@@ -1603,23 +1590,6 @@ __global__ void __launch_bounds__(kT, 1) k_res_reverse(ResJob<KT> one, const Res
         v.amps[i] = x0;
         v.lam[i] = l0;
         ++pairs;
-      }
-    }
-    if (Net::kGrid && n_scan + recs > v.L) {
-      // No room beside dropped entries for the records: they leave first.
-      __syncthreads();
-      const unsigned int dead = s_dead;
-      __syncthreads();  // (read by every thread before the records change it)
-      if (dead) {
-        const unsigned int kept = res_squeeze(v, n_scan);
-        if (tid == 0) {
-          s_tail = kept;
-          s_dead = 0u;
-          if (sweep) scanned += n_scan - kept;
-        }
-        n_scan = kept;
-        res_rehash(v, kept, cnt);
-        ++compactions;
       }
     }
     // The records of factor k - 1: a key that is still stored was dropped.
