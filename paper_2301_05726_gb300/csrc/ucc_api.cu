@@ -677,8 +677,8 @@ ucc_status resident_tape(ucc_ctx* c, const Counters& h, const ResGeom& g) {
 }
 
 // What a resident run that starts with `live` determinants in table s needs before
-// its first factor (record: in a gradient): tape, inboxes, and room in the table
-// for what it may write back.  *ready = false: not all of that can be had.  Then no memory is
+// its first factor (record: in a gradient): room in the table for what it may write
+// back, inboxes, and tape.  *ready = false: not all of that can be had.  Then no memory is
 // kept for it: a launch per factor, which runs instead, needs little at first.
 // The contents of s and of the tape are lost.
 template <class KT>
@@ -688,9 +688,9 @@ ucc_status resident_prepare(ucc_ctx* c, TableSet& s, unsigned long long live, bo
   if (c->K == 0 || !resident_shape(c, &g) || !res_room(live, g)) return UCC_OK;
   const unsigned long long cap = resident_cap(c, g);
   ResNet<KT> net{};
-  ucc_status r = record ? resident_tape(c, Counters{}, g) : UCC_OK;
+  ucc_status r = s.cur.cap_n < cap ? s.cur.allocate(cap, slots_for(cap)) : UCC_OK;
   if (r == UCC_OK) r = resident_net<KT>(c, g, &net);
-  if (r == UCC_OK && s.cur.cap_n < cap) r = s.cur.allocate(cap, slots_for(cap));
+  if (r == UCC_OK && record) r = resident_tape(c, Counters{}, g);
   if (r == UCC_ENOMEM) {
     s.cur.release();
     dfree(c->d_res_key);
