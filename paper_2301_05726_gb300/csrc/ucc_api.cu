@@ -126,6 +126,9 @@ struct TableSet {
   // Whether cur's slot array and filter index its entries.  A resident pass
   // leaves entries only; ensure_hash builds the hash when a kernel needs it.
   bool hash_valid = true;
+  // Whether the last run_factors ran all its factors resident: the reverse sweep
+  // goes back over the same tables, so it fits where they did.
+  bool ran_resident = false;
   void release() {
     cur.release();
     spare.release();
@@ -984,13 +987,13 @@ ucc_status resident_forward(ucc_ctx* c, TableSet& s, double eps, bool record, in
   return UCC_OK;
 }
 
-// The reverse of the factors [k0, k1) on table s in one resident launch, if it
-// fits; *done says so.
+// The reverse of the factors [k0, k1) on table s in one resident launch, if their
+// tables fit; *done says so.
 template <class KT>
 ucc_status resident_reverse(ucc_ctx* c, TableSet& s, int k0, int k1, bool* done) {
   *done = false;
   ResGeom g{};
-  if (!resident_shape(c, &g) || s.cur.cap_n < resident_cap(c, g)) return UCC_OK;
+  if (!s.ran_resident || !resident_shape(c, &g) || s.cur.cap_n < resident_cap(c, g)) return UCC_OK;
   if (!res_room(s.h_cnt->n_tail - s.h_cnt->n_dead, g)) return UCC_OK;
   ResNet<KT> net{};
   const ucc_status n = resident_net<KT>(c, g, &net);
@@ -1024,7 +1027,8 @@ ucc_status run_factors(ucc_ctx* c, TableSet& s, double eps, bool record, int k0,
   UCC_TRY(read_counters(c, s));
   int k = k0;
   UCC_TRY(resident_forward<KT>(c, s, eps, record, &k, k1));
-  if (k == k1) return UCC_OK;
+  s.ran_resident = k == k1;
+  if (s.ran_resident) return UCC_OK;
   UCC_TRY(ensure_hash<KT>(c, s));
   // Room for the next factor, as after every stop.  A table that a resident pass
   // of the segment before this one left needs it too: that pass leaves no more

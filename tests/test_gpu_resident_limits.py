@@ -208,3 +208,14 @@ def test_dropped_entries_near_the_room(torch_cuda):
     E, g = ctx.gradient()
     assert_gradient((E, g), p)
     assert ctx.stats()["forward_launches"] == 1 and ctx.stats()["reverse_launches"] == 1
+
+
+@pytest.mark.parametrize("stride", [0, 15])
+def test_no_reverse_pass_over_tables_that_do_not_fit(torch_cuda, stride):
+    # The final state fits the GPU, a table on the way does not: the reverse sweep of the
+    # factors around it takes a launch each, without a resident one before them.
+    p = dataclasses.replace(doubling(20, extra=[(0, 1, 20, 21), (2, 3, 22, 23)]), n_max=1_000_000, n_cut=100_000)
+    ctx = context(p, checkpoint_stride=stride)
+    assert_gradient(ctx.gradient(), p, checkpoint_stride=stride)
+    # (with segments the first fifteen factors run resident: one launch)
+    assert ctx.stats()["reverse_launches"] == (p.n_exc if stride == 0 else p.n_exc - 15 + 1)
