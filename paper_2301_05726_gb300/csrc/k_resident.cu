@@ -56,6 +56,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "ucc_steps.cuh"
 
@@ -1761,8 +1762,20 @@ ResLimits find_limits() {
 }  // namespace
 
 ResLimits res_limits(int key_words) {
-  static const ResLimits one = find_limits<unsigned long long>(), two = find_limits<Key128>();
-  return key_words == 2 ? two : one;
+  // kept per device: SM counts and cluster sizes may differ between them
+  constexpr int kDevices = 64;
+  static std::mutex mutex;
+  static ResLimits found[2][kDevices];
+  static bool have[2][kDevices];
+  const int w = key_words == 2 ? 1 : 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return ResLimits{};
+  std::lock_guard<std::mutex> lock(mutex);
+  if (!have[w][dev]) {
+    found[w][dev] = w ? find_limits<Key128>() : find_limits<unsigned long long>();
+    have[w][dev] = true;
+  }
+  return found[w][dev];
 }
 
 bool res_room(unsigned long long entries, const ResGeom& g) {
