@@ -402,7 +402,7 @@ def batch_leg(args):
 
     probs = jobs(range(256))
     ctxs = [UCCContext(p) for p in probs]
-    batch_run(ctxs, 1e-8, with_grad=True)  # warm-up (tunes probe width and tiles once)
+    batch_run(ctxs, 1e-8, with_grad=True)  # warm-up
     torch.cuda.synchronize()
     t0 = time.perf_counter()
     E, _ = batch_run(ctxs, 1e-8, with_grad=True)
@@ -417,7 +417,7 @@ def batch_leg(args):
            "jobs_cut": sum(x["cut"] > 0 for x in st)}
     for c in ctxs:
         c.close()
-    # a sample of jobs: the batch vs one job at a time (the one-job path, host-driven cuts)
+    # a sample of jobs: the batch vs one job at a time (the one-job path, itself resident)
     sample = list(range(0, 256, 32))
     sp = jobs(sample)
     sc = [UCCContext(p) for p in sp]

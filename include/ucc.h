@@ -121,7 +121,10 @@ typedef struct {
                                     whole-GPU resident launches; 0 = none */
   int32_t batch_tiles;       /* ucc_batch_run: 32-entry tiles a warp takes per
                                 visit of a job (1, 2, 4 or 8); 0 = autotuned.
-                                Read from the first job. */
+                                Read from the first job.  A width set here keeps
+                                jobs that fit a thread-block cluster in the
+                                persistent launches too (by default they run
+                                resident, a cluster each) */
   int32_t energy_route;      /* ucc_energy / ucc_gradient: 0 = by buckets of
                                 shared cores when their records fit device
                                 memory, else per connection; 1 = per
@@ -169,7 +172,9 @@ typedef struct {
   int64_t recompute_created;   /* gradient: entries created while recomputing segments */
   int64_t forward_launches;    /* forward factor launches (incl. recomputation) */
   int64_t reverse_launches;    /* reverse factor launches */
-  int64_t probe_width;         /* lanes per hash probe in use (fixed or autotuned) */
+  int64_t probe_width;         /* lanes per hash probe in use (fixed or autotuned);
+                                  1 for a batch's resident jobs, which probe no
+                                  global hash in their factor steps */
   int64_t reverse_scanned;     /* entries scanned by the reverse sweep's factor steps */
   int64_t reverse_compactions; /* compactions of the table during the reverse sweep */
   double apply_ms;          /* device time of the last forward pass */
@@ -178,7 +183,8 @@ typedef struct {
   double forward_kernel_ms; /* device time of the forward factor launches alone */
   double reverse_kernel_ms; /* device time of the reverse factor launches alone */
   int64_t batch_tiles;      /* ucc_batch_run: 32-entry tiles a warp takes per
-                               visit of a job (fixed by the autotuner) */
+                               visit of a job (fixed or autotuned); 1 for
+                               resident jobs, which take no tiles */
   double cut_ms;            /* device time of the Methods-section cuts (selection,
                                compaction, rehash) of the last forward pass */
   double rebuild_ms;        /* device time of the other compactions and growths */
