@@ -1788,7 +1788,14 @@ bool res_cluster_shape(unsigned long long most, int key_words, int max_ctas, boo
   // instructions of 16 cycles a warp: its SMs are worth more than its barriers cost
   // (a factor at 100, 1,225 and 3,136 determinants: 5.5, 4.9 and 4.9 us with the
   // clusters of the other runs, 4.8, 4.7 and 4.7 with sixteen; the whole GPU: 6.0,
-  // 5.7, 5.8).
+  // 5.7, 5.8).  Without entropies the other size matters too, a batch's jobs in
+  // flight: 24 gradients over 3,136 determinants take 4.9, 7.0 and 10.6 ms with 4, 8
+  // and 16 CTAs each, while one by itself gains little from more (us per factor,
+  // forward and reverse: 225 determinants 3.0 and 3.4 with 1, 3.1 and 3.2 with 4, 3.0
+  // and 2.9 with 8; 441: 3.1 and 3.6, 3.1 and 3.5, 3.0 and 3.2; 1,568: 3.4 and 4.4, 3.3
+  // and 3.8, 3.1 and 3.5; 4,900: 3.7 and 4.6 with 4, 3.3 and 4.0 with 8, 3.3 and 3.9
+  // with 16; 7,056: 3.3 and 4.0 with 8, 3.4 and 4.0 with 16; 10,584: 3.6 and 4.2, 3.3
+  // and 3.8).
   int ctas = entropy ? kMaxC : most <= 512 ? 1 : most <= 2048 ? 4 : most <= 6144 ? 8 : 16;
   ctas = std::min(ctas, max_ctas);
   for (; ctas <= max_ctas; ctas *= 2) {

@@ -1734,8 +1734,11 @@ ucc_status batch_resident(const std::vector<int>& idx, ucc_ctx* const* jobs, dou
   });
   unsigned long long most = 1;
   for (int x : order) most = std::max(most, most_entries(jobs[x]));
-  // Clusters of eight keep twice as many jobs in flight as clusters of
-  // sixteen, which pays from ten jobs on (nine large clusters fill the GPU).
+  // Clusters of eight, where they hold the largest job (tables of up to some
+  // 10,700), keep twice as many jobs in flight as clusters of sixteen: 4, 9, 14 and 24
+  // gradients over 7,056 determinants take 2.7, 3.2, 3.7 and 7.0 ms with eight, 2.7,
+  // 5.4, 6.0 and 11.4 with sixteen.  (The line could lie a job lower.  N_MAX 8,000
+  // takes sixteen for up to 16,000 determinants in any case.)
   const int lim = res_limits(1).cluster;
   ResGeom g{};
   if (!(n > 9 && res_cluster_shape(most, 1, std::min(lim, 8), false, &g)) &&
@@ -2508,6 +2511,7 @@ ucc_status ucc_batch_run(int n_jobs, ucc_ctx* const* jobs, double eps, double* E
   // one; the rest share the persistent launches.
   std::vector<int> together, resident, alone;
   for (int j = 0; j < n_jobs; ++j) {
+    jobs[j]->res_gave_up = false;
     if (batch_resident_ok(jobs[j], jobs[0]->opt) && resident.size() < (size_t)kMaxBatchJobs)
       resident.push_back(j);
     else if (batch_capacity(jobs[j]) == 0 || together.size() >= (size_t)kMaxBatchJobs)

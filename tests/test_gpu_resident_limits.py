@@ -175,6 +175,22 @@ def test_a_wait_that_runs_out(torch_cuda, wide):
         assert np.array_equal(x, y)
 
 
+def test_a_wait_that_ran_out_ends_with_its_call(torch_cuda):
+    # A whole-GPU launch of the last call gave up; a batch over the same context, with a
+    # cut that a cluster holds, runs resident (the persistent launches would size its
+    # table at three times N_MAX).
+    from paper_2301_05726_gb300.api import batch_run
+    p = synth.make_problem(77, 12, 4, 4, 0.08).prefix(120)
+    ctx = context(p, batch_wait_ms=50, batch_test_skip_block=2)
+    ctx.apply()
+    assert ctx.stats()["forward_launches"] > p.n_exc
+    cut = dict(n_max=2000, n_cut=1000)
+    ctx.set_options(batch_wait_ms=0, batch_test_skip_block=0, **cut)
+    E, grads = batch_run([ctx], 0.0)
+    assert ctx.stats()["capacity_entries"] != 3 * cut["n_max"]
+    assert_gradient((E[0], grads[0]), p, **cut)
+
+
 def test_dropped_entries_near_the_room(torch_cuda):
     # 714,208 determinants, near the 760,000 that the GPU holds, then factors of angle
     # pi/2: each moves some 5 % of them, so that what it leaves behind is dropped.
