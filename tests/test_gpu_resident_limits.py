@@ -235,3 +235,11 @@ def test_no_reverse_pass_over_tables_that_do_not_fit(torch_cuda, stride):
     assert_gradient(ctx.gradient(), p, checkpoint_stride=stride)
     # (with segments the first fifteen factors run resident: one launch)
     assert ctx.stats()["reverse_launches"] == (p.n_exc if stride == 0 else p.n_exc - 15 + 1)
+
+
+def test_the_first_table_of_a_small_problem(torch_cuda):
+    # 36 determinants in the sector: the table has the size of any first one.
+    p = synth.make_problem(77, 4, 2, 2, 0.08)
+    ctx = context(p)
+    ctx.apply()
+    assert ctx.stats()["n_det"] <= 36 and ctx.stats()["capacity_entries"] == 4096
