@@ -1099,6 +1099,8 @@ ucc_status run_factors(ucc_ctx* c, TableSet& s, double eps, bool record, int k0,
       Counters known = h;
       if (h.cut_pending) {
         const unsigned long long before = h.n_tail - h.n_dead, kept = (unsigned long long)c->opt.n_cut;
+        // (the room kept ahead of a factor is for its own drops)
+        if (record) UCC_TRY(ensure_tape(c, h.tape_n + (before - kept)));
         UCC_TRY(cut_rebuild<KT>(c, s, record, resume - 1));
         known.n_tail = kept;
         known.n_dead = 0;
